@@ -130,6 +130,14 @@ typedef struct bt_info {
  * bits above the smallest key are below j (32-byte keys: bits of the 8 bytes
  * after the bytes all keys share).
  *
+ * Beside the image, in an allocation of its own that bt_info does not count,
+ * the device keeps a walk index: the keys and values once more in 64-byte
+ * entries under 32-byte nodes, through which batches are searched as given
+ * (see bt_search_opts.sort_bits).  It takes about 20 bytes per 64-bit key
+ * and value (12 for 32-bit ones, 70 per 32-byte key) and is left out when
+ * that is more than a quarter of the free device memory; searches are then
+ * partitioned and descend the tree as bt_sort_bits says.
+ *
  * Errors: BT_ERR_ARG, BT_ERR_FANOUT, BT_ERR_UNSORTED, BT_ERR_DUPLICATE,
  * BT_ERR_NOMEM, BT_ERR_CUDA.  *out is set only on BT_OK.
  */
@@ -161,11 +169,17 @@ typedef struct bt_search_opts {
     /* Bits of the bucket number the batch is partitioned on before the
      * descent (Sec. IV-A sorts the batch so that queries for one node are
      * adjacent; see bt_sort_batch for the order obtained): -1 lets the
-     * library choose (none below 786432 queries -- 393216 for 32-byte
+     * library choose, 0 skips the partition, 1..21 forces that many bits
+     * (larger values mean 21).  A batch that is not forced goes through the
+     * tree's walk index as given, the faster way at every size, unless the
+     * tree has none, d_fetch_counts is set, or another descent than the
+     * pipelined one with the binary-search rank has been chosen for it
+     * (bt_tree_set_staging, bt_tree_set_lane_queries, bt_tree_set_descent);
+     * then -1 partitions on
+     * bt_sort_bits bits (none below 786432 queries -- 393216 for 32-byte
      * keys -- and none for a tree whose device image is at most a quarter of
      * the L2: the partition pays for itself only when the batch is large and
-     * leaf blocks do not stay in the L2 between batches), 0 skips the
-     * partition, 1..21 forces that many bits (larger values mean 21). */
+     * leaf blocks do not stay in the L2 between batches). */
     int32_t sort_bits;
     /* If non-NULL: device array of `height` counters to which the search
      * adds, per level, how many node key blocks it fetched -- the quantity
@@ -550,7 +564,9 @@ bt_status bt_check_timeouts(void);
  * for every combination of warps per block {4, 8, 16}, pinned bytes
  * {0, 16384, 49152} and descent design (pipelined with inner levels read
  * through L1 or staged; synchronous with cp.async or bulk-copy staging; two
- * queries per lane); keep the fastest.  *out receives the tree built with
+ * queries per lane); keep the fastest.  The pipelined settings search the
+ * sample through the walk index, on which none of them bears: they are timed
+ * once per fanout, at 8 warps and 16384 pinned bytes.  *out receives the tree built with
  * the best fanout and launch parameters applied, *best the choice and its
  * time.  A sample with fewer 32-query chunks per SM than a warps-per-block
  * setting runs the pipelined descent in smaller blocks whatever that setting

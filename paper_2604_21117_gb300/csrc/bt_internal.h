@@ -80,6 +80,21 @@ struct PaperTree {
     uint32_t pin_bytes;   // bytes of those levels (a prefix of the array)
 };
 
+// The walk index of a tree (walk.cuh), passed to kernels by value.
+constexpr int kWalkLevels = 12;
+struct WalkDev {
+    const unsigned char *top;      // segments' largest keys, a binary tree in breadth-first order
+    const unsigned char *nodes;    // 32-byte nodes, level 0 (one node per segment) first
+    const unsigned char *entries;  // 64-byte entries
+    uint64_t off[kWalkLevels];     // byte offset of each level in nodes
+    uint64_t n;                    // keys
+    uint64_t kmin32[4], kmax32[4]; // 32-byte keys: the smallest and largest key
+    int p0;                        // 32-byte keys: bytes all keys share; the word walked follows them
+    int levels;                    // levels of nodes
+    int top_bits;                  // depth of the binary tree (0: one segment, no top)
+    uint32_t top_bytes;
+};
+
 // Whole top levels (never the leaves) whose bytes fit `budget`, root first.
 void set_pin_levels(DevTree &d, const bt_info &info, uint32_t budget);
 
@@ -107,6 +122,8 @@ struct bt_tree {
     float l2_hit_ratio;
     btgb::PaperTree paper;  // valid once d_paper is set (bt_paper_layout_build)
     void *d_paper;
+    btgb::WalkDev walk;  // valid while d_walk is set
+    void *d_walk;        // the walk index (null: not built)
 };
 
 struct bt_model {

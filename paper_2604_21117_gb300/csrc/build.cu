@@ -17,6 +17,7 @@
 #include <vector>
 
 #include "bt_internal.h"
+#include "descent.cuh"
 
 namespace btgb {
 
@@ -508,6 +509,12 @@ extern "C" bt_status bt_build(const void *h_keys, const void *h_vals, uint64_t n
     d.split_off = kb == 32 ? static_cast<unsigned char *>(t->d_image) + split_off_offset : nullptr;
     d.split_R = reinterpret_cast<const uint16_t *>(static_cast<unsigned char *>(t->d_image) + split_R_offset);
     t->info.d_image = t->d_image;
+    e = walk_build(t, s);
+    if (e != cudaSuccess) {
+        set_error_detail("walk index", e);
+        bt_free(t);
+        return BT_ERR_CUDA;
+    }
     *out = t;
     return BT_OK;
 }
@@ -515,6 +522,7 @@ extern "C" bt_status bt_build(const void *h_keys, const void *h_vals, uint64_t n
 extern "C" void bt_free(bt_tree *t)
 {
     if (!t) return;
+    if (t->d_walk) cudaFree(t->d_walk);
     if (t->d_image) cudaFree(t->d_image);
     if (t->d_paper) cudaFree(t->d_paper);
     delete t;

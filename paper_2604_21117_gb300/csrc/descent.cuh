@@ -312,6 +312,14 @@ cudaError_t descend_synchronous(const DescendArgs &a, cudaStream_t s);
 cudaError_t descend_paper_layout(const DevTree &t, const PaperTree &p, const void *q, const uint32_t *qidx,
                                  const void *recs, uint64_t nq, void *out_v, uint8_t *out_f, cudaStream_t s);
 
+// Builds the walk index of a tree whose image is on the device, in an
+// allocation of its own.  Leaves the tree without one (and returns
+// cudaSuccess) when the index would take more than a quarter of the free
+// device memory, or the key count exceeds what its node numbers hold.
+cudaError_t walk_build(bt_tree *tree, cudaStream_t s);
+// Search of a batch as given through the walk index.
+cudaError_t walk_search(const bt_tree *tree, const void *q, uint64_t nq, void *out_v, uint8_t *out_f, cudaStream_t s);
+
 // Grid of a persistent descent: enough blocks for the chunks, at most one
 // full wave of resident blocks.
 cudaError_t persistent_grid(const void *kern, int threads, int smem, uint64_t units_per_block, uint64_t units,
@@ -331,6 +339,7 @@ static inline cudaError_t take_wait_counters(unsigned *timeouts, unsigned *pendi
     return e;
 }
 cudaError_t take_wait_counters_pipelined(unsigned *timeouts, unsigned *pending);
+cudaError_t take_wait_counters_walk(unsigned *timeouts, unsigned *pending);
 cudaError_t take_wait_counters_synchronous(unsigned *timeouts, unsigned *pending);
 
 }  // namespace btgb

@@ -51,6 +51,16 @@ __device__ __forceinline__ uint64_t bytes_be64(uint64_t x)
     return (static_cast<uint64_t>(__byte_perm(lo, 0, 0x0123)) << 32) | __byte_perm(hi, 0, 0x0123);
 }
 
+// 8 bytes of a 32-byte key from byte p on (p <= 24), as a big-endian number.
+__device__ __forceinline__ uint64_t key32_window(const Key32 &k, int p)
+{
+    const int j = p >> 3, s = (p & 7) * 8;
+    // selects: an indexed word would put the key in local memory
+    const uint64_t hi = j == 0 ? k.w[0] : (j == 1 ? k.w[1] : (j == 2 ? k.w[2] : k.w[3]));
+    const uint64_t lo = j == 0 ? k.w[1] : (j == 1 ? k.w[2] : (j == 2 ? k.w[3] : 0ull));
+    return s ? (hi << s) | (lo >> (64 - s)) : hi;
+}
+
 // How each key type is read from a query array, and its all-ones value.
 template <typename K>
 struct KeyOps {

@@ -190,15 +190,6 @@ __device__ __forceinline__ uint32_t part_bucket(const PartSmem<K> &S, const Part
     return (c << pn.r) | static_cast<uint32_t>(x);
 }
 
-// 8 bytes of a 32-byte key from byte p on (p <= 24), as a big-endian number.
-__device__ __forceinline__ uint64_t key32_window(const Key32 &k, int p)
-{
-    const int j = p >> 3, s = (p & 7) * 8;
-    const uint64_t hi = k.w[j];
-    const uint64_t lo = j < 3 ? k.w[j + 1] : 0ull;
-    return s ? (hi << s) | (lo >> (64 - s)) : hi;
-}
-
 // f(q) for 32-byte keys.
 __device__ __forceinline__ uint32_t part_bucket(const PartSmem<Key32> &S, const PartNorm<Key32> &pn, const Key32 &q)
 {

@@ -1,7 +1,8 @@
 // Batched level-wise B+ tree point search on GB300 (sm_103a): the search
 // entry points.
 //
-// One search is (Sec. IV-A, IV-F):
+// A batch that is not forced into the partition is searched as given through
+// the tree's walk index (walk.cuh).  Otherwise one search is (Sec. IV-A, IV-F):
 //   1. an on-device partition of (query, input position) pairs by a bucket
 //      number monotone in the key (part_sort.cuh), so that queries routed
 //      to the same node end up adjacent (the paper's sorted batch);
@@ -56,6 +57,16 @@ static cudaError_t descend(const bt_tree *tree, const void *q, const uint32_t *q
 {
     const DescendArgs a{view ? view : &tree->dev, tree, q, qidx, recs, nq, out_v, out_f, fetch, nullptr, nullptr};
     return descend_any(a, s);
+}
+
+// Whether a search that forces no partition goes through the tree's walk
+// index: the tree has one, and its descent is the pipelined one with the
+// binary-search rank, the defaults (the synchronous designs, two queries per
+// lane and the ballot rank are run as chosen).
+static bool walk_takes(const bt_tree *tree)
+{
+    const DevTree &t = tree->dev;
+    return tree->d_walk && t.staging == BT_STAGE_PIPELINED && t.lane_queries == 1 && t.rank_ballot == 0;
 }
 
 template <typename V>
@@ -122,8 +133,8 @@ static bool arrays_aligned(const DevTree &t, const void *keys, const void *qidx,
            (reinterpret_cast<uintptr_t>(vals) & (va - 1)) == 0;
 }
 
-// Queries per batch from which the automatic choice partitions the batch,
-// for trees larger than a quarter of the L2 (DevTree::sort_pays).  Measured
+// Queries per batch from which the automatic choice partitions a batch that
+// does not go through the walk index, for trees larger than a quarter of the L2 (DevTree::sort_pays).  Measured
 // on uint64 trees at fanout 32: on 2^24 keys the unsorted descent is faster
 // up to 2^19 queries (53 against 61 us), the sorted search from 2^20 (86
 // against 90 us); on 4 * 10^6 keys (67 MB) likewise (49 against 52 us at 2^19,
@@ -382,6 +393,19 @@ extern "C" bt_status bt_search_batch_ex(const bt_tree *tree, const void *d_queri
         return BT_OK;
     }
 
+    if (opts ? opts->sort_bits <= 0 && !opts->d_fetch_counts && walk_takes(tree) : walk_takes(tree)) {
+        e = opts && opts->phase_event ? cudaEventRecord(static_cast<cudaEvent_t>(opts->phase_event), s) : cudaSuccess;
+        if (e != cudaSuccess) {
+            set_error_detail("phase event", e);
+            return BT_ERR_CUDA;
+        }
+        e = walk_search(tree, d_queries, nq, d_out_vals, d_out_found, s);
+        if (e != cudaSuccess) {
+            set_error_detail("walk launch", e);
+            return BT_ERR_CUDA;
+        }
+        return BT_OK;
+    }
     const PartPlan pp = plan_partition(t, opts ? opts->sort_bits : -1, nq);
     const void *q = d_queries;
     const uint32_t *qidx = nullptr;
@@ -612,6 +636,7 @@ extern "C" bt_status bt_check_timeouts(void)
         if (e == cudaSuccess && v) e = cudaMemcpyToSymbol(g_part_timeouts, &zero, sizeof(zero));
         timeouts += v;
     }
+    if (e == cudaSuccess) e = take_wait_counters_walk(&timeouts, &pending);
     if (e == cudaSuccess) e = take_wait_counters_synchronous(&timeouts, &pending);
     if (e != cudaSuccess) {
         set_error_detail("timeout counters", e);

@@ -4,7 +4,8 @@
 // built and the sample searched with every combination of warps per block
 // {4, 8, 16}, shared-memory pin budget {0, 16 KB, 48 KB} and descent design
 // (pipelined with inner levels through L1 or staged; synchronous with
-// cp.async or bulk-copy staging; two queries per lane); the fastest
+// cp.async or bulk-copy staging; two queries per lane); with the pipelined
+// design the sample goes through the tree's walk index; the fastest
 // combination (median of timed repetitions, CUDA events on the caller's
 // stream) wins and its tree is returned with those settings applied.
 #include <cuda_runtime.h>
@@ -111,7 +112,7 @@ extern "C" bt_status bt_autotune(const void *h_keys, const void *h_vals, uint64_
     }
     const uint64_t sample_per_sm = ((nsample + 31) / 32 + static_cast<uint64_t>(sms > 0 ? sms : 1) - 1) /
                                    static_cast<uint64_t>(sms > 0 ? sms : 1);
-    constexpr uint32_t kDefaultWarps = 8;
+    constexpr uint32_t kDefaultWarps = 8, kDefaultPin = 16384;
     bt_tree *keep = nullptr;
     bt_tune b{0, 0, 0, 0, 1, 0, 0.0f};
     for (uint32_t m : fanouts) {
@@ -135,6 +136,10 @@ extern "C" bt_status bt_autotune(const void *h_keys, const void *h_vals, uint64_
                 static const uint32_t kStage[5] = {BT_STAGE_PIPELINED, BT_STAGE_PIPELINED, BT_STAGE_CP_ASYNC,
                                                    BT_STAGE_BULK, BT_STAGE_CP_ASYNC};
                 const uint32_t sm = kStage[cfg], lq = cfg == 4 ? 2u : 1u, inner = cfg == 1 ? 1u : 0u;
+                // the pipelined settings search the sample through the walk index,
+                // which none of the launch parameters touch: timed once
+                if (sm == BT_STAGE_PIPELINED && t->d_walk && (inner || w != kDefaultWarps || p != kDefaultPin))
+                    continue;
                 if (sm == BT_STAGE_PIPELINED && sample_per_sm < w && w != kDefaultWarps) continue;
                 bt_tree_set_launch(t, w, p);
                 bt_tree_set_staging(t, sm);

@@ -1,0 +1,83 @@
+"""Batches searched as given through the walk index, against the CPU oracle
+and against the partitioned descent, at the sizes where the index changes
+shape: one entry, a full and an overfull top, one node more per level, ragged
+last entries; for 32-byte keys also words that tie."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+from paper_2604_21117_gb300 import workloads as W
+from oracle import OracleTree
+from oracle.bytes_keys import OracleBytesTree
+import pins
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def bt():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2604_21117_gb300 import build_lib
+    build_lib.build()
+    from paper_2604_21117_gb300 import btree
+    return btree
+
+
+def _same(tree, o, q):
+    import torch
+    ov, of, _, _ = o.search(q)
+    for sb in (-1, 0, 12):  # the walk index twice, the partition and descent once
+        v, f = tree.search(torch.from_numpy(np.ascontiguousarray(q)).cuda(), sort_bits=sb)
+        assert np.array_equal(v.cpu().numpy().astype(np.uint64), ov)
+        assert np.array_equal(f.cpu().numpy(), of)
+
+
+# entries hold 32 / max(widths) keys, the top 2^13 segments (2^14 for 32-bit
+# keys), a node 5 children (9 for 32-bit keys)
+@pytest.mark.parametrize("kw,vw,n", [
+    (64, 64, 1), (64, 64, 4), (64, 64, 5), (64, 64, 4 * 8192), (64, 64, 4 * 8192 + 1), (64, 64, 4 * 5 * 8192),
+    (64, 64, 4 * 5 * 8192 + 1), (64, 64, 4 * 25 * 8192 + 3), (64, 32, 4 * 8192 + 2), (32, 64, 4 * 16384 + 1),
+    (32, 32, 7), (32, 32, 8 * 16384), (32, 32, 8 * 16384 + 1), (32, 32, 8 * 9 * 16384 + 5)])
+@pytest.mark.parametrize("nq", [1, 33, 152 * 1024 + 33])
+def test_index_shape_boundaries(bt, kw, vw, n, nq):
+    keys = W.uniform_keys(n, kw, seed=900 + n)
+    vals = W.rng(901).integers(0, 2**vw, size=n, dtype=np.uint64).astype(W.key_dtype(vw))
+    tree = bt.BTree(keys, vals, 16)
+    o = OracleTree(keys, vals, 16, val_bits=vw)
+    g = W.rng(902 + nq)
+    probes = pins.probe_queries(keys, kw, g) if nq > 1000 else W.make_queries(keys, nq, 0.7, seed=nq, width_bits=kw)
+    _same(tree, o, np.resize(probes, nq).astype(W.key_dtype(kw)))
+
+
+def test_all_ones_key_stored_and_not(bt):
+    top = 2**64 - 1
+    for keys in ([1, 2, 3, top], [1, 2, 3, top - 1, top], [5], [top], [0, top]):
+        keys = np.array(keys, np.uint64)
+        tree = bt.BTree(keys, np.arange(10, 10 + keys.size, dtype=np.uint64), 8)
+        o = OracleTree(keys, np.arange(10, 10 + keys.size, dtype=np.uint64), 8)
+        _same(tree, o, np.array([top, top - 1, 0, 1, 4, 5], np.uint64))
+
+
+@pytest.mark.parametrize("n", [1, 2, 8192, 8193, 5 * 8192 + 1])
+@pytest.mark.parametrize("tie", [0, 7, 5000])
+def test_byte_keys_with_tied_words(bt, n, tie):
+    """Runs of `tie` keys that share the 8 bytes the index walks and differ
+    only later, so that the search has to go on from the first of a run;
+    queries inside runs, at their ends, between them and outside all keys."""
+    g = W.rng(910 + n + tie)
+    keys = g.integers(0, 256, size=(n, 32), dtype=np.uint8)
+    if tie:
+        keys[:, :8] = g.integers(0, 256, size=(n // tie + 1, 8), dtype=np.uint8)[np.arange(n) // tie]
+    keys = W._sort_rows(keys)
+    vals = W.rank_values(keys.shape[0], 64)
+    tree = bt.BTree(keys, vals, 16)
+    o = OracleBytesTree(keys, vals, 16)
+    q = W.make_byte_queries(keys, 3001, 0.7, seed=911)
+    near = keys[g.integers(0, keys.shape[0], size=500)].copy()
+    near[:, 31] ^= 1
+    ends = np.stack([keys[0], keys[-1], np.zeros(32, np.uint8), np.full(32, 255, np.uint8)])
+    _same(tree, o, np.concatenate([q, near, ends]))
+    o.close()
