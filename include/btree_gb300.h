@@ -376,7 +376,10 @@ typedef struct bt_forest bt_forest;
  * ones are staged per warp (the synchronous designs and inner-staged
  * pipelined design) or read lane by lane through L1 (the pipelined design).
  * Warps per block default to the setting of the tree with the most keys,
- * the pin budget to 32 KB.  The trees must outlive the forest.
+ * the pin budget to 32 KB.  A forest none of whose trees is staged per warp,
+ * and all of whose trees have a walk index (see bt_build), searches them
+ * through it instead, in chunks of 32 queries and blocks of its own shape:
+ * those settings then have no effect.  The trees must outlive the forest.
  * Errors: BT_ERR_ARG, BT_ERR_NOMEM, BT_ERR_CUDA. */
 bt_status bt_forest_create(const bt_tree *const *trees, uint32_t count, bt_forest **out);
 

@@ -340,6 +340,7 @@ static inline cudaError_t take_wait_counters(unsigned *timeouts, unsigned *pendi
 }
 cudaError_t take_wait_counters_pipelined(unsigned *timeouts, unsigned *pending);
 cudaError_t take_wait_counters_walk(unsigned *timeouts, unsigned *pending);
+cudaError_t take_wait_counters_forest(unsigned *timeouts, unsigned *pending);
 cudaError_t take_wait_counters_synchronous(unsigned *timeouts, unsigned *pending);
 
 }  // namespace btgb

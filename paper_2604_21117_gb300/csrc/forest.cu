@@ -1,5 +1,9 @@
 // Many batches over several resident trees in one persistent launch.
 //
+// A forest whose trees all have a walk index, none a model and none staged
+// per warp is searched by forest_walk.cu's kernel; what follows is the
+// descent that serves the others.
+//
 // A "forest" is a table of built trees sharing key and value widths
 // (fanouts may differ), each with its own launch settings: the top levels
 // pinned in shared memory, queries per lane, and whether the levels below
@@ -42,6 +46,10 @@ struct bt_forest {
     uint32_t stage_mode;   // 0: each tree's tuned design, 1: all through L1, 2: all staged
     uint32_t pin_total;    // bytes of the pinned levels actually applied
     uint32_t stage_bytes;  // per warp, 0 when no tree is staged
+    btgb::ForestWalk *d_walk;  // table of the walk kernel
+    bool walk;             // work lists go to the walk kernel (every tree has a walk index or is empty, no
+                           // model, no tree staged per warp)
+    uint32_t walk_top;     // bytes of the tops it copies to shared memory
     int model_set;         // kModelNone (no model), kModelPL (PL models only), kModelMLP (any model)
 };
 
@@ -55,11 +63,11 @@ constexpr int kForestStageBytes = 4096;  // per warp, staged trees: 8..64 node b
 constexpr uint32_t kForestSmemList = 64;  // work lists up to this long are read from shared memory
 constexpr uint32_t kForestPinMax = 98304;
 constexpr int kForestSmemMax = 200 * 1024;
-
-__host__ __device__ inline bool forest_desc_ok(const bt_batch_desc &bd, uint32_t ntrees, uint64_t nq)
-{
-    return bd.tree < ntrees && bd.offset <= nq && bd.count <= nq - bd.offset;
-}
+// Tops of a forest's trees in shared memory.  10,000 batches over trees of
+// 10^3, 10^5, 10^6 and 2 * 10^7 uint64 keys (146 KB of tops): 58.9 us with all
+// of them there, 71.7 with 96 KB (the largest tree's top through L1), 68.9
+// with none.
+constexpr uint32_t kWalkTopBudget = 160 * 1024;
 
 __host__ __device__ inline uint32_t forest_desc_chunks(const bt_batch_desc &bd, uint32_t ntrees, uint64_t nq,
                                                        int lq)
@@ -456,6 +464,9 @@ cudaError_t forest_run(const bt_forest *f, const bt_batch_desc *b, uint32_t nb, 
                        uint32_t host_chunks, uint32_t *plan_ws, const void *q, uint64_t nq, void *ov, uint8_t *of,
                        uint32_t warps, cudaStream_t s, ForestDone done)
 {
+    if (f->walk && (cs || nb <= kForestWalkList))
+        return forest_walk_run(f->d_walk, f->count, f->walk_top, f->key_bytes, f->val_bytes, b, nb, cs, host_chunks, q,
+                               nq, ov, of, s, done);
     if (f->key_bytes == 8) {
         if (f->val_bytes == 8) return forest_launch_t<uint64_t, uint64_t>(f, b, nb, cs, host_chunks, plan_ws, q, nq, ov, of, warps, s, done);
         return forest_launch_t<uint64_t, uint32_t>(f, b, nb, cs, host_chunks, plan_ws, q, nq, ov, of, warps, s, done);
@@ -469,7 +480,8 @@ void forest_chunks(const bt_forest *f, const bt_batch_desc *b, uint32_t nb, uint
     uint32_t run = 0;
     for (uint32_t i = 0; i < nb; ++i) {
         cs[i] = run;
-        run += forest_desc_chunks(b[i], f->count, ~0ull, b[i].tree < f->count ? f->h_tab[b[i].tree].lq : 1);
+        run += forest_desc_chunks(b[i], f->count, ~0ull,
+                                  !f->walk && b[i].tree < f->count ? f->h_tab[b[i].tree].lq : 1);
     }
     cs[nb] = run;
 }
@@ -531,6 +543,35 @@ static void forest_table(bt_forest *f)
         if (k == kModelPL && f->model_set == kModelNone) f->model_set = kModelPL;
     }
     f->stage_bytes = any_staged ? static_cast<uint32_t>(kForestStageBytes) : 0u;
+    f->walk = !any_staged && f->model_set == kModelNone;
+    for (uint32_t i = 0; i < n; ++i)
+        if (f->trees[i]->dev.height > 0 && !f->trees[i]->d_walk) f->walk = false;
+}
+
+// The walk kernel's table: the tops that fit kWalkTopBudget have a place in
+// shared memory, the smallest first (a top read through L1 costs its tree
+// most when it is small and would always have fitted).
+static std::vector<ForestWalk> walk_table(bt_forest *f)
+{
+    std::vector<ForestWalk> tab(f->count, ForestWalk{});
+    std::vector<uint32_t> order(f->count);
+    for (uint32_t i = 0; i < f->count; ++i) {
+        order[i] = i;
+        if (f->trees[i]->d_walk) tab[i].w = f->trees[i]->walk;
+        tab[i].top_off = kNoTop;
+        // in units of one probe of the top: a sector from the L2 costs about
+        // six, the entry two, the rest of a chunk's work about ten
+        tab[i].cost = 22u + static_cast<uint32_t>(tab[i].w.top_bits + 6 * tab[i].w.levels);
+    }
+    std::sort(order.begin(), order.end(),
+              [&](uint32_t a, uint32_t b) { return tab[a].w.top_bytes < tab[b].w.top_bytes; });
+    f->walk_top = 0;
+    for (uint32_t i : order) {
+        if (f->walk_top + tab[i].w.top_bytes > kWalkTopBudget) break;
+        tab[i].top_off = f->walk_top;
+        f->walk_top += tab[i].w.top_bytes;
+    }
+    return tab;
 }
 
 static bt_status forest_upload(bt_forest *f)
@@ -539,6 +580,9 @@ static bt_status forest_upload(bt_forest *f)
     cudaError_t e = cudaDeviceSynchronize();  // no search may be reading the old table
     if (e == cudaSuccess)
         e = cudaMemcpy(f->d_tab, f->h_tab.data(), sizeof(ForestTree) * f->count, cudaMemcpyHostToDevice);
+    const std::vector<ForestWalk> walk = walk_table(f);
+    if (e == cudaSuccess)
+        e = cudaMemcpy(f->d_walk, walk.data(), sizeof(ForestWalk) * f->count, cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
         set_error_detail("forest table", e);
         return BT_ERR_CUDA;
@@ -565,6 +609,7 @@ static bt_status forest_create(const bt_tree *const *trees, const bt_model *cons
     bt_forest *f = new (std::nothrow) bt_forest;
     if (!f) return BT_ERR_NOMEM;
     f->d_tab = nullptr;
+    f->d_walk = nullptr;
     f->count = count;
     f->trees.assign(trees, trees + count);
     f->models.assign(count, nullptr);
@@ -581,14 +626,17 @@ static bt_status forest_create(const bt_tree *const *trees, const bt_model *cons
     f->lane_mode = 0;
     f->stage_mode = 0;
     cudaError_t e = cudaMalloc(&f->d_tab, sizeof(ForestTree) * count);
+    if (e == cudaSuccess) e = cudaMalloc(&f->d_walk, sizeof(ForestWalk) * count);
     if (e != cudaSuccess) {
         set_error_detail("forest table", e);
+        cudaFree(f->d_tab);
         delete f;
         return e == cudaErrorMemoryAllocation ? BT_ERR_NOMEM : BT_ERR_CUDA;
     }
     const bt_status st = forest_upload(f);
     if (st != BT_OK) {
         cudaFree(f->d_tab);
+        cudaFree(f->d_walk);
         delete f;
         return st;
     }
@@ -612,6 +660,7 @@ extern "C" void bt_forest_free(bt_forest *f)
 {
     if (!f) return;
     cudaFree(f->d_tab);
+    cudaFree(f->d_walk);
     delete f;
 }
 
@@ -761,6 +810,7 @@ extern "C" bt_status bt_forest_bad_batches(uint64_t *out)
         const unsigned long long zero = 0;
         e = cudaMemcpyToSymbol(g_bt_bad_batches, &zero, sizeof(zero));
     }
+    if (e == cudaSuccess) e = forest_walk_take_bad(&v);
     if (e != cudaSuccess) {
         set_error_detail("rejected-batch counter", e);
         return BT_ERR_CUDA;

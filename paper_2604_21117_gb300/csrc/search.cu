@@ -637,6 +637,7 @@ extern "C" bt_status bt_check_timeouts(void)
         timeouts += v;
     }
     if (e == cudaSuccess) e = take_wait_counters_walk(&timeouts, &pending);
+    if (e == cudaSuccess) e = take_wait_counters_forest(&timeouts, &pending);
     if (e == cudaSuccess) e = take_wait_counters_synchronous(&timeouts, &pending);
     if (e != cudaSuccess) {
         set_error_detail("timeout counters", e);

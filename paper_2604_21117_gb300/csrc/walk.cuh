@@ -111,6 +111,15 @@ __device__ __forceinline__ uint32_t walk_segment(const W *top, int bits, W q)
     return k - (1u << bits);
 }
 
+// The same from the top in global memory, through L1.
+template <typename W>
+__device__ __forceinline__ uint32_t walk_segment_l1(const unsigned char *top, int bits, W q)
+{
+    uint32_t k = 1;
+    for (int i = 0; i < bits; ++i) k = 2u * k + (ld_key(reinterpret_cast<const W *>(top) + k) < q ? 1u : 0u);
+    return k - (1u << bits);
+}
+
 // The entry of q from its segment: the first entry whose largest key (32-byte
 // keys: word) is not below q, or the last one.
 template <typename W>

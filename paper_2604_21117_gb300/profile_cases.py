@@ -4,6 +4,7 @@
     python -m paper_2604_21117_gb300.profile_cases keys32 [sorted|full]
     python -m paper_2604_21117_gb300.profile_cases crossover
     python -m paper_2604_21117_gb300.profile_cases shapes
+    python -m paper_2604_21117_gb300.profile_cases walk [keys batch fanout]
 
 forest: the multi-tree batching workload -- trees of 10^3, 10^5, 10^6 and
 2*10^7 uniform uint64 keys at fanout 32, a work list of 10,000 batches whose
@@ -26,6 +27,9 @@ shapes: the descent of 2^20 queries partitioned on 20 bits over 2^24 uniform
 uint64 keys at fanout 32 (four batches in turn), at 4, 8 and 16 warps per
 block and 1 to 8 resident blocks per SM (bt_tree_set_corun; "max" = as many
 as fit); medians of 60 launches.
+
+walk: six searches of a batch as given (default 2^20 queries at 90% hits over
+2^24 uniform uint64 keys, fanout 32), four batches in turn.
 
 Each prints its CUDA-event times; the inputs come from workloads.py with
 fixed seeds.
@@ -215,9 +219,33 @@ def shapes(steps: int = 60) -> None:
     tree.close()
 
 
+def walk(n: int = 1 << 24, B: int = 1 << 20, m: int = 32) -> None:
+    import torch
+    from . import build_lib
+    build_lib.build()
+    from . import btree as bt
+    from . import workloads as W
+    keys = W.uniform_keys(n, 64, seed=W.SEED_BASE + 2)
+    tree = bt.BTree(keys, W.rank_values(n, 64), m)
+    nb = tree.workspace_bytes(B)
+    ws = torch.empty(nb, dtype=torch.uint8, device="cuda")
+    v, f = tree.alloc_outputs(B)
+    s = torch.cuda.current_stream()
+    qs = [torch.from_numpy(W.make_queries(keys, B, 0.9, seed=W.SEED_BASE + 2 + 1000 * (i + 1), width_bits=64)).cuda()
+          for i in range(4)]
+    for it in range(6):
+        e0, e1 = _events()
+        e0.record(s)
+        bt.bt_search_batch(tree.handle, qs[it % 4], B, v, f, ws, nb, s)
+        e1.record(s)
+        torch.cuda.synchronize()
+        print(f"walk {it}: {1000 * e0.elapsed_time(e1):.1f} us")
+    tree.close()
+
+
 def main(argv=None) -> int:
     argv = sys.argv[1:] if argv is None else argv
-    if not argv or argv[0] not in ("forest", "keys32", "crossover", "shapes"):
+    if not argv or argv[0] not in ("forest", "keys32", "crossover", "shapes", "walk"):
         print(__doc__)
         return 2
     if argv[0] == "forest":
@@ -226,6 +254,8 @@ def main(argv=None) -> int:
         keys32(*argv[1:2])
     elif argv[0] == "crossover":
         crossover()
+    elif argv[0] == "walk":
+        walk(*(int(x) for x in argv[1:4]))
     else:
         shapes()
     return 0

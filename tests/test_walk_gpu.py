@@ -81,3 +81,49 @@ def test_byte_keys_with_tied_words(bt, n, tie):
     ends = np.stack([keys[0], keys[-1], np.zeros(32, np.uint8), np.full(32, 255, np.uint8)])
     _same(tree, o, np.concatenate([q, near, ends]))
     o.close()
+
+
+@pytest.mark.parametrize("ntrees,nb", [(1, 1), (3, 31), (3, 33), (40, 700), (4, 65_536), (4, 65_537)])
+def test_work_lists_through_the_walk_kernel(bt, ntrees, nb):
+    """Lists shorter and longer than a row, longer than the kernel plans
+    itself (then the descent's), more trees than its table and its tops have
+    room for, empty trees and batches, and bad entries."""
+    import torch
+    g = W.rng(920 + nb)
+    sizes = [0 if i % 7 == 6 else int(3 * 8 ** (1 + i % 5)) for i in range(ntrees)]
+    keysets = [W.uniform_keys(n, 64, seed=921 + i) for i, n in enumerate(sizes)]
+    trees = [bt.BTree(k, W.rank_values(k.size, 64), 16) for k in keysets]
+    forest = bt.bt_forest_create([t.handle for t in trees])
+    desc = np.zeros(nb, bt.BATCH_DESC_DTYPE)
+    desc["tree"] = g.integers(0, ntrees, size=nb)
+    counts = g.choice([0, 1, 5, 31, 32, 33, 70], size=nb)
+    desc["count"], desc["offset"] = counts, np.cumsum(counts) - counts
+    total = max(1, int(counts.sum()))
+    q = g.integers(0, 2**64, size=total, dtype=np.uint64)
+    want_v, want_f = np.full(total, 5, np.uint64), np.full(total, 9, np.uint8)
+    for i, k in enumerate(keysets):
+        rows = np.flatnonzero(desc["tree"] == i)
+        at = np.concatenate([np.arange(o, o + c) for o, c in zip(desc["offset"][rows], counts[rows])] or
+                            [np.empty(0)]).astype(np.int64)
+        if k.size:
+            hit = g.random(at.size) < 0.7
+            q[at[hit]] = k[g.integers(0, k.size, size=int(hit.sum()))]
+        pos = np.searchsorted(k, q[at]) if k.size else np.zeros(at.size, np.int64)
+        found = (pos < k.size) & (k[np.minimum(pos, max(k.size - 1, 0))] == q[at]) if k.size else np.zeros(at.size, bool)
+        want_v[at], want_f[at] = np.where(found, pos.astype(np.uint64), np.uint64(2**64 - 1)), found
+    bad = np.flatnonzero(counts > 0)[: 2 if nb > 30 else 0]  # rejected: nothing is written for them
+    for b, (field, value) in zip(bad, [("tree", ntrees), ("offset", total + 1)]):
+        o, c = int(desc["offset"][b]), int(counts[b])
+        want_v[o:o + c], want_f[o:o + c] = 5, 9
+        desc[field][b] = value
+    dq = torch.from_numpy(q).cuda()
+    v = torch.full((total,), 5, dtype=torch.int64, device="cuda")
+    f = torch.full((total,), 9, dtype=torch.uint8, device="cuda")
+    wsb = bt.bt_forest_workspace_bytes(nb)
+    ws = torch.empty(wsb, dtype=torch.uint8, device="cuda")
+    bt.bt_forest_bad_batches()
+    bt.bt_forest_search(forest, torch.from_numpy(desc.view(np.uint8)).cuda(), nb, dq, v, f, ws, wsb)
+    torch.cuda.synchronize()
+    assert bt.bt_forest_bad_batches() == len(bad)
+    assert np.array_equal(v.cpu().numpy().view(np.uint64), want_v) and np.array_equal(f.cpu().numpy(), want_f)
+    bt.bt_forest_free(forest)
