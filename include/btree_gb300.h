@@ -833,8 +833,10 @@ bt_status bt_learned_descend_sorted(const bt_tree *tree, const bt_model *model, 
                                     const uint32_t *d_index, uint64_t nq, void *d_out_vals,
                                     uint8_t *d_out_found, unsigned long long *d_stats, bt_stream stream);
 
-/* bt_search_batch with the model (sort, then the learned descent); same
- * workspace, results identical to bt_search_batch. */
+/* bt_search_batch with the model, results identical to it: the batch as given
+ * through the tree's walk index, the model's window in place of the search
+ * of its top (a window the index's separators do not prove is not used);
+ * without a walk index sort, then the learned descent.  Same workspace. */
 bt_status bt_learned_search_batch(const bt_tree *tree, const bt_model *model, const void *d_queries,
                                   uint64_t nq, void *d_out_vals, uint8_t *d_out_found, void *d_workspace,
                                   uint64_t ws_bytes, bt_stream stream);

@@ -197,32 +197,8 @@ __global__ void BT_DESCEND_REGS k_descend(
     const unsigned char *top = static_cast<const unsigned char *>(t.keys[0]);
     for (uint32_t i = threadIdx.x * 16u; i < pin_bytes; i += blockDim.x * 16u) cp_async16_ca(pin + i, top + i);
     // The model's parameters, copied once per block when they fit.
-    const uint64_t *mb = md.b;
-    const float *minv = md.inv_w, *mslope = md.slope, *micpt = md.icpt, *mmlp = md.mlp;
-    if constexpr (LEARN) {
-        if (mbytes) {
-            if constexpr (MODEL == kModelPL) {
-                const uint32_t S = md.segments;
-                uint64_t *sb = reinterpret_cast<uint64_t *>(msm);
-                float *sf = reinterpret_cast<float *>(msm + S * 8u);
-                for (uint32_t i = threadIdx.x; i < S; i += blockDim.x) {
-                    sb[i] = md.b[i];
-                    sf[i] = md.inv_w[i];
-                    sf[S + i] = md.slope[i];
-                    sf[2 * S + i] = md.icpt[i];
-                }
-                mb = sb;
-                minv = sf;
-                mslope = sf + S;
-                micpt = sf + 2 * S;
-            } else {
-                float *sp = reinterpret_cast<float *>(msm);
-                for (uint32_t i = threadIdx.x; i < static_cast<uint32_t>(kMlpParams); i += blockDim.x)
-                    sp[i] = md.mlp[i];
-                mmlp = sp;
-            }
-        }
-    }
+    ModelView mv{};
+    if constexpr (LEARN) mv = model_to_smem<MODEL>(md, msm);
     // the batch (and the outputs) belong to the previous kernel until it is
     // done; the copies above stay in flight meanwhile
     pdl_wait();
@@ -284,14 +260,8 @@ __global__ void BT_DESCEND_REGS k_descend(
                 // windows (unsorted batches) are checked lane by lane in
                 // global memory.
                 const uint32_t L = md.leaves;
-                uint32_t hat;
-                if constexpr (MODEL == kModelPL)
-                    hat = leaf_from_pred(pl_predict(mb, minv, mslope, micpt, md.segments, static_cast<uint64_t>(key)), L);
-                else
-                    hat = model_leaf(md, mb, minv, mslope, micpt, mmlp, static_cast<uint64_t>(key));
-                const uint32_t er = __ldg(md.errs + err_range(hat, L));
-                const uint32_t lo = hat > er ? hat - er : 0u;
-                const uint32_t hi = (static_cast<uint64_t>(hat) + er < L) ? hat + er : L - 1;
+                uint32_t lo, hi;
+                model_window<MODEL>(md, mv, static_cast<uint64_t>(key), lo, hi);
                 uint32_t wlo = __reduce_min_sync(0xffffffffu, lo);
                 if (wlo > 0) --wlo;
                 const uint32_t whi = __reduce_max_sync(0xffffffffu, hi);

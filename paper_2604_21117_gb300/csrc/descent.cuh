@@ -283,8 +283,70 @@ constexpr uint32_t kModelSmemSegments = 512;
 __host__ __device__ inline uint32_t model_smem_bytes(const ModelDev &m)
 {
     if (m.kind == kModelPL) return m.segments <= kModelSmemSegments ? (m.segments * 20u + 15u) / 16u * 16u : 0u;
-    if (m.kind == kModelMLP) return (kMlpParams * 4u + 15u) / 16u * 16u;
+    if (m.kind == kModelMLP) return (kMlpStage1 * 12u + kMlpParams * 4u + 15u) / 16u * 16u;
     return 0u;
+}
+
+// Where a block finds a model's parameters: in its shared memory when they
+// fit there, else in global memory.
+struct ModelView {
+    const uint64_t *b;
+    const float *inv_w, *slope, *icpt, *mlp;
+};
+
+// Copies the parameters of a model that fits (model_smem_bytes > 0) to msm
+// (16-byte aligned); every thread of the block takes part, a block barrier
+// has to follow.
+template <int MODEL>
+__device__ __forceinline__ ModelView model_to_smem(const ModelDev &md, unsigned char *msm)
+{
+    ModelView v{md.b, md.inv_w, md.slope, md.icpt, md.mlp};
+    if (model_smem_bytes(md) == 0) return v;
+    if constexpr (MODEL == kModelPL) {
+        const uint32_t S = md.segments;
+        uint64_t *sb = reinterpret_cast<uint64_t *>(msm);
+        float *sf = reinterpret_cast<float *>(msm + S * 8u);
+        for (uint32_t i = threadIdx.x; i < S; i += blockDim.x) {
+            sb[i] = md.b[i];
+            sf[i] = md.inv_w[i];
+            sf[S + i] = md.slope[i];
+            sf[2 * S + i] = md.icpt[i];
+        }
+        v.b = sb;
+        v.inv_w = sf;
+        v.slope = sf + S;
+        v.icpt = sf + 2 * S;
+    } else {
+        uint64_t *sb = reinterpret_cast<uint64_t *>(msm);
+        float *sf = reinterpret_cast<float *>(msm + kMlpStage1 * 8u);
+        float *sp = sf + kMlpStage1;
+        for (uint32_t i = threadIdx.x; i < kMlpStage1; i += blockDim.x) {
+            sb[i] = md.b[i];
+            sf[i] = md.inv_w[i];
+        }
+        for (uint32_t i = threadIdx.x; i < static_cast<uint32_t>(kMlpParams); i += blockDim.x) sp[i] = md.mlp[i];
+        v.b = sb;
+        v.inv_w = sf;
+        v.mlp = sp;
+    }
+    return v;
+}
+
+// The leaf a model predicts for q, and the window of leaves [lo, hi] its
+// error bound allows.
+template <int MODEL>
+__device__ __forceinline__ void model_window(const ModelDev &md, const ModelView &v, uint64_t q, uint32_t &lo,
+                                             uint32_t &hi)
+{
+    const uint32_t L = md.leaves;
+    uint32_t hat;
+    if constexpr (MODEL == kModelPL)
+        hat = leaf_from_pred(pl_predict(v.b, v.inv_w, v.slope, v.icpt, md.segments, q), L);
+    else
+        hat = leaf_from_pred(__fmul_rn(mlp_forward(v.mlp, mlp_x_rank(v.b, v.inv_w, q)), static_cast<float>(L - 1)), L);
+    const uint32_t er = __ldg(md.errs + err_range(hat, L));
+    lo = hat > er ? hat - er : 0u;
+    hi = (static_cast<uint64_t>(hat) + er < L) ? hat + er : L - 1;
 }
 
 // ------------------------------------------------------- host interface
@@ -317,8 +379,10 @@ cudaError_t descend_paper_layout(const DevTree &t, const PaperTree &p, const voi
 // cudaSuccess) when the index would take more than a quarter of the free
 // device memory, or the key count exceeds what its node numbers hold.
 cudaError_t walk_build(bt_tree *tree, cudaStream_t s);
-// Search of a batch as given through the walk index.
-cudaError_t walk_search(const bt_tree *tree, const void *q, uint64_t nq, void *out_v, uint8_t *out_f, cudaStream_t s);
+// Search of a batch as given through the walk index; md: with a model of the
+// tree (integer keys).
+cudaError_t walk_search(const bt_tree *tree, const void *q, uint64_t nq, void *out_v, uint8_t *out_f, cudaStream_t s,
+                        const ModelDev *md = nullptr);
 
 // Grid of a persistent descent: enough blocks for the chunks, at most one
 // full wave of resident blocks.

@@ -104,18 +104,28 @@ __device__ __forceinline__ float mlp_x(uint64_t q, uint64_t kmin, uint64_t kmax,
     return __fmul_rn(__double2float_rn(__ull2double_rn(c - kmin)), inv_range);
 }
 
-// Network output for input x (parameters p, any address space).
+// Network output for input x (parameters p, any address space, 16-byte
+// aligned).  A lane evaluates the whole network: the second layer's rows are
+// read four weights at a time, so that a warp's loads (one broadcast each)
+// stay below its multiplications.
 __device__ __forceinline__ float mlp_forward(const float *p, float x)
 {
     float h1[kMlpH];
 #pragma unroll
     for (int j = 0; j < kMlpH; ++j) h1[j] = fmaxf(fmaf(p[kOffW1 + j], x, p[kOffB1 + j]), 0.0f);
     float y = p[kOffB3];
-#pragma unroll 4
+#pragma unroll 8
     for (int j = 0; j < kMlpH; ++j) {
+        const float4 *w = reinterpret_cast<const float4 *>(p + kOffW2 + j * kMlpH);
         float z = p[kOffB2 + j];
 #pragma unroll
-        for (int k = 0; k < kMlpH; ++k) z = fmaf(p[kOffW2 + j * kMlpH + k], h1[k], z);
+        for (int k = 0; k < kMlpH / 4; ++k) {
+            const float4 v = w[k];
+            z = fmaf(v.x, h1[4 * k], z);
+            z = fmaf(v.y, h1[4 * k + 1], z);
+            z = fmaf(v.z, h1[4 * k + 2], z);
+            z = fmaf(v.w, h1[4 * k + 3], z);
+        }
         y = fmaf(p[kOffW3 + j], fmaxf(z, 0.0f), y);
     }
     return y;

@@ -599,6 +599,14 @@ extern "C" bt_status bt_learned_search_batch(const bt_tree *tree, const bt_model
     if (!d_workspace || ws_bytes < w.total || (reinterpret_cast<uintptr_t>(d_workspace) & 255u))
         return BT_ERR_WORKSPACE;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+    if (tree->d_walk) {
+        const cudaError_t we = walk_search(tree, d_queries, nq, d_out_vals, d_out_found, s, &model->dev);
+        if (we != cudaSuccess) {
+            set_error_detail("learned walk launch", we);
+            return BT_ERR_CUDA;
+        }
+        return BT_OK;
+    }
     const PartPlan pp = plan_partition(t, -1, nq);
     const void *q = d_queries;
     const uint32_t *qidx = nullptr;

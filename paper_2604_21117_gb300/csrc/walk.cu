@@ -204,7 +204,18 @@ cudaError_t walk_build(bt_tree *t, cudaStream_t s)
 
 // --------------------------------------------------------------- search
 
-constexpr int kWalkThreads = 1024;
+template <int MODEL>
+constexpr int walk_threads()
+{
+    return MODEL == kModelMLP ? 512 : 1024;  // the network's hidden layer stays in registers
+}
+
+// A model and what turns its window of leaves into one of segments.
+struct WalkModel {
+    ModelDev md;
+    uint64_t leaf_base, leaf_rem;  // keys per leaf, leaves with one more
+    uint32_t span;                 // entries per segment
+};
 
 // One query per lane, one block per SM; every block takes a contiguous run
 // of 32-query chunks of the batch, its warps chunk by chunk in turn, the
@@ -224,10 +235,14 @@ constexpr int kWalkThreads = 1024;
 // The kernel does not trigger the launch of its successor: blocks started
 // early pair up on the SMs that drain first, and the batch then waits for
 // those (300,007 uint32 queries: 15.0 us with the trigger, 8.6 without).
-template <typename K, typename V>
-__global__ void __launch_bounds__(kWalkThreads) k_walk(const WalkDev w, const RawOf<K> *__restrict__ q, uint32_t nq,
-                                                       V *__restrict__ out_v, uint8_t *__restrict__ out_f,
-                                                       uint32_t wait_polls)
+//
+// MODEL: the learned search.  The model's window of leaves, as a range of
+// segments, takes the place of the top's binary search where the separators
+// around it prove it; the walk below is the same.
+template <typename K, typename V, int MODEL>
+__global__ void __launch_bounds__(walk_threads<MODEL>())
+    k_walk(const WalkDev w, const WalkModel m, const RawOf<K> *__restrict__ q, uint32_t nq, V *__restrict__ out_v,
+           uint8_t *__restrict__ out_f, uint32_t wait_polls)
 {
     using W = typename WalkWord<K>::type;
     extern __shared__ __align__(128) unsigned char smem[];
@@ -238,6 +253,8 @@ __global__ void __launch_bounds__(kWalkThreads) k_walk(const WalkDev w, const Ra
         mbar_arrive_expect_tx(&bar, w.top_bytes);
         if (w.top_bytes) bulk_g2s(smem, w.top, w.top_bytes, &bar);
     }
+    ModelView mv{};
+    if constexpr (MODEL != kModelNone) mv = model_to_smem<MODEL>(m.md, smem + w.top_bytes);
     pdl_wait();
     const uint32_t chunks = (nq + 31) / 32;
     const uint32_t c1 = static_cast<uint32_t>(static_cast<uint64_t>(chunks) * (blockIdx.x + 1) / gridDim.x);
@@ -249,7 +266,7 @@ __global__ void __launch_bounds__(kWalkThreads) k_walk(const WalkDev w, const Ra
     };
     K next = KeyOps<K>::ones();
     if (c < c1) next = load(c);
-    __syncthreads();  // the barrier is initialised
+    __syncthreads();  // the barrier is initialised, the model copied
     if (!mbar_wait_warp(&bar, 0, wait_polls)) {
         mbar_give_up(&bar, 0, static_cast<int>(lane));
         return;
@@ -270,7 +287,20 @@ __global__ void __launch_bounds__(kWalkThreads) k_walk(const WalkDev w, const Ra
         } else {
             word = key;
         }
-        const uint32_t seg = walk_segment<W>(reinterpret_cast<const W *>(smem), w.top_bits, word);
+        const W *top = reinterpret_cast<const W *>(smem);
+        uint32_t seg;
+        if constexpr (MODEL == kModelNone) {
+            seg = walk_segment<W>(top, w.top_bits, word);
+        } else {
+            constexpr uint32_t G = walk_group(sizeof(K), sizeof(V));
+            uint32_t lo, hi;
+            model_window<MODEL>(m.md, mv, static_cast<uint64_t>(key), lo, hi);
+            // first key of leaf lo, last key of leaf hi, as entries, as segments
+            const uint64_t r0 = lo * m.leaf_base + (lo < m.leaf_rem ? lo : m.leaf_rem);
+            const uint64_t r1 = (hi + 1ull) * m.leaf_base + (hi + 1ull < m.leaf_rem ? hi + 1ull : m.leaf_rem) - 1;
+            seg = walk_segment_in<W>(top, w.top_bits, static_cast<uint32_t>(r0 / G) / m.span,
+                                     static_cast<uint32_t>(r1 / G) / m.span, word);
+        }
         V val;
         bool hit = walk_lookup<K, V>(w, walk_entry<W>(w, seg, word), key, val);
         if (!in) {
@@ -285,27 +315,39 @@ __global__ void __launch_bounds__(kWalkThreads) k_walk(const WalkDev w, const Ra
     }
 }
 
-template <typename K, typename V>
-static cudaError_t walk_launch(const WalkDev &w, const void *q, uint64_t nq, void *out_v, uint8_t *out_f,
-                               cudaStream_t s)
+template <typename K, typename V, int MODEL>
+static cudaError_t walk_launch(const bt_tree *t, const ModelDev *md, const void *q, uint64_t nq, void *out_v,
+                               uint8_t *out_f, cudaStream_t s)
 {
-    auto kern = k_walk<K, V>;
+    auto kern = k_walk<K, V, MODEL>;
+    const WalkDev &w = t->walk;
+    constexpr int kMaxTop = static_cast<int>(sizeof(typename WalkWord<K>::type)) << walk_top_bits(sizeof(K));
+    constexpr int kMaxModel = MODEL == kModelNone ? 0 : static_cast<int>(kModelSmemSegments) * 20;
     int sms = 0;
     cudaError_t e = dev_sm_count(&sms);
-    if (e == cudaSuccess)
-        e = ensure_dyn_smem(reinterpret_cast<const void *>(kern),
-                            static_cast<int>(sizeof(typename WalkWord<K>::type)) << walk_top_bits(sizeof(K)));
+    if (e == cudaSuccess) e = ensure_dyn_smem(reinterpret_cast<const void *>(kern), kMaxTop + kMaxModel);
     if (e != cudaSuccess) return e;
-    // one block per SM with as many warps as its share of the chunks, at most 32
+    WalkModel m;
+    memset(&m, 0, sizeof(m));
+    if (MODEL != kModelNone) {
+        const int leaf = t->dev.height - 1;
+        m.md = *md;
+        m.leaf_base = t->dev.cbase[leaf];
+        m.leaf_rem = t->dev.crem[leaf];
+        m.span = 1;
+        for (int l = 0; l < w.levels; ++l) m.span *= walk_fan(static_cast<int>(sizeof(K)));
+    }
+    // one block per SM with as many warps as its share of the chunks
+    constexpr uint64_t kWarps = walk_threads<MODEL>() / 32;
     const uint64_t chunks = (nq + 31) / 32, n = static_cast<uint64_t>(sms > 0 ? sms : 1);
     const uint64_t per_sm = (chunks + n - 1) / n;
-    const uint64_t warps = per_sm < kWalkThreads / 32 ? per_sm : kWalkThreads / 32;
+    const uint64_t warps = per_sm < kWarps ? per_sm : kWarps;
     const uint64_t grid = (chunks + warps - 1) / warps < n ? (chunks + warps - 1) / warps : n;
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
     cfg.gridDim = dim3(static_cast<unsigned>(grid));
     cfg.blockDim = dim3(static_cast<unsigned>(warps * 32));
-    cfg.dynamicSmemBytes = w.top_bytes;
+    cfg.dynamicSmemBytes = w.top_bytes + (MODEL == kModelNone ? 0u : model_smem_bytes(m.md));
     cfg.stream = s;
     cudaLaunchAttribute attr;
     memset(&attr, 0, sizeof(attr));
@@ -313,22 +355,34 @@ static cudaError_t walk_launch(const WalkDev &w, const void *q, uint64_t nq, voi
     attr.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, w, static_cast<const RawOf<K> *>(q), static_cast<uint32_t>(nq),
+    return cudaLaunchKernelEx(&cfg, kern, w, m, static_cast<const RawOf<K> *>(q), static_cast<uint32_t>(nq),
                               static_cast<V *>(out_v), out_f, first_wait_polls());
 }
 
-cudaError_t walk_search(const bt_tree *t, const void *q, uint64_t nq, void *out_v, uint8_t *out_f, cudaStream_t s)
+template <typename K, typename V>
+static cudaError_t walk_model(const bt_tree *t, const ModelDev *md, const void *q, uint64_t nq, void *out_v,
+                              uint8_t *out_f, cudaStream_t s)
 {
-    const WalkDev &w = t->walk;
+    if constexpr (sizeof(K) <= 8) {
+        if (md && md->kind == kModelPL) return walk_launch<K, V, kModelPL>(t, md, q, nq, out_v, out_f, s);
+        if (md) return walk_launch<K, V, kModelMLP>(t, md, q, nq, out_v, out_f, s);
+    }
+    return walk_launch<K, V, kModelNone>(t, md, q, nq, out_v, out_f, s);
+}
+
+cudaError_t walk_search(const bt_tree *t, const void *q, uint64_t nq, void *out_v, uint8_t *out_f, cudaStream_t s,
+                        const ModelDev *md)
+{
     const int kb = t->dev.key_bytes;
+    const bool v8 = t->dev.val_bytes == 8;
     if (kb == 32)
-        return t->dev.val_bytes == 8 ? walk_launch<Key32, uint64_t>(w, q, nq, out_v, out_f, s)
-                                     : walk_launch<Key32, uint32_t>(w, q, nq, out_v, out_f, s);
+        return v8 ? walk_model<Key32, uint64_t>(t, md, q, nq, out_v, out_f, s)
+                  : walk_model<Key32, uint32_t>(t, md, q, nq, out_v, out_f, s);
     if (kb == 8)
-        return t->dev.val_bytes == 8 ? walk_launch<uint64_t, uint64_t>(w, q, nq, out_v, out_f, s)
-                                     : walk_launch<uint64_t, uint32_t>(w, q, nq, out_v, out_f, s);
-    return t->dev.val_bytes == 8 ? walk_launch<uint32_t, uint64_t>(w, q, nq, out_v, out_f, s)
-                                 : walk_launch<uint32_t, uint32_t>(w, q, nq, out_v, out_f, s);
+        return v8 ? walk_model<uint64_t, uint64_t>(t, md, q, nq, out_v, out_f, s)
+                  : walk_model<uint64_t, uint32_t>(t, md, q, nq, out_v, out_f, s);
+    return v8 ? walk_model<uint32_t, uint64_t>(t, md, q, nq, out_v, out_f, s)
+              : walk_model<uint32_t, uint32_t>(t, md, q, nq, out_v, out_f, s);
 }
 
 cudaError_t take_wait_counters_walk(unsigned *timeouts, unsigned *pending)

@@ -111,6 +111,32 @@ __device__ __forceinline__ uint32_t walk_segment(const W *top, int bits, W q)
     return k - (1u << bits);
 }
 
+// Separator of sorted rank r of the top (all-ones from the last segment on).
+template <typename W>
+__device__ __forceinline__ W walk_top_at(const W *top, int bits, uint32_t r)
+{
+    const int t = __ffs(static_cast<int>(r + 1)) - 1;  // the node's height over the bottom
+    return top[(1u << (bits - 1 - t)) + ((r + 1) >> (t + 1))];
+}
+
+// The same segment when [s0, s1] is believed to hold it: proven by the
+// separators on both sides and searched inside, else the whole top searched.
+template <typename W>
+__device__ __forceinline__ uint32_t walk_segment_in(const W *top, int bits, uint32_t s0, uint32_t s1, W q)
+{
+    const uint32_t last = (1u << bits) - 1;  // position behind the separators
+    if ((s0 > 0 && !(walk_top_at(top, bits, s0 - 1) < q)) || (s1 < last && walk_top_at(top, bits, s1) < q))
+        return walk_segment(top, bits, q);
+    while (s0 < s1) {
+        const uint32_t mid = (s0 + s1) / 2;
+        if (walk_top_at(top, bits, mid) < q)
+            s0 = mid + 1;
+        else
+            s1 = mid;
+    }
+    return s0;
+}
+
 // The same from the top in global memory, through L1.
 template <typename W>
 __device__ __forceinline__ uint32_t walk_segment_l1(const unsigned char *top, int bits, W q)

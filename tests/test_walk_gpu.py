@@ -127,3 +127,29 @@ def test_work_lists_through_the_walk_kernel(bt, ntrees, nb):
     assert bt.bt_forest_bad_batches() == len(bad)
     assert np.array_equal(v.cpu().numpy().view(np.uint64), want_v) and np.array_equal(f.cpu().numpy(), want_f)
     bt.bt_forest_free(forest)
+
+
+@pytest.mark.parametrize("kind", ["pl1", "pl", "pl_many", "mlp"])
+@pytest.mark.parametrize("kw,n", [(64, 3), (64, 200), (64, 4 * 8192 + 5), (64, 400_000), (32, 8 * 16384 + 9)])
+def test_learned_search_through_the_walk(bt, kind, kw, n):
+    """Models whose windows span one leaf, many segments and the whole tree
+    (one line over lognormal keys), parameters in shared and in global memory."""
+    import torch
+    keys = W.lognormal_mixture_keys(n, seed=930) if kw == 64 else W.uniform_keys(n, kw, seed=930)
+    vals = W.rank_values(n, 64)
+    tree = bt.BTree(keys, vals, 32)
+    o = OracleTree(keys, vals, 32)
+    if kind == "mlp":
+        m = bt.bt_model_train(tree.handle, bt.BT_MODEL_MLP, h_init=W.mlp_init_params(931), steps=20, batch=1024,
+                              lr=2e-3, seed=932)
+    else:
+        m = bt.bt_model_train(tree.handle, bt.BT_MODEL_PL, segments={"pl1": 1, "pl": 64, "pl_many": 2000}[kind])
+    for nq in (1, 4099, 152 * 512 + 7):
+        q = W.make_queries(keys, nq, 0.7, seed=933 + nq, width_bits=kw)
+        q[:1] = keys[-1]
+        ov, of, _, _ = o.search(q)
+        v, f = tree.alloc_outputs(nq)
+        ws, nb = tree.alloc_workspace(nq)
+        bt.bt_learned_search_batch(tree.handle, m, torch.from_numpy(q).cuda(), nq, v, f, ws, nb)
+        assert np.array_equal(v.cpu().numpy(), ov) and np.array_equal(f.cpu().numpy(), of)
+    bt.bt_model_free(m)
