@@ -153,3 +153,37 @@ def test_learned_search_through_the_walk(bt, kind, kw, n):
         bt.bt_learned_search_batch(tree.handle, m, torch.from_numpy(q).cuda(), nq, v, f, ws, nb)
         assert np.array_equal(v.cpu().numpy(), ov) and np.array_equal(f.cpu().numpy(), of)
     bt.bt_model_free(m)
+
+
+@pytest.mark.parametrize("kw,vw", [(64, 64), (32, 64), (64, 32), (256, 64)])
+@pytest.mark.parametrize("where", ["pinned", "pageable", "queries", "results", "misaligned", "shared"])
+def test_host_buffers_in_place_and_copied(bt, kw, vw, where):
+    """Host buffers used in place (page-locked), copied (pageable, off their
+    alignment, results over the queries' memory), and some of each."""
+    import torch
+    n, nq = 30_000, 5003
+    if kw == 256:
+        keys = W.byte_keys(n, 32, seed=940)
+        q = W.make_byte_queries(keys, nq, 0.7, seed=941)
+        o = OracleBytesTree(keys, W.rank_values(n, vw), 16)
+    else:
+        keys = W.uniform_keys(n, kw, seed=940)
+        q = W.make_queries(keys, nq, 0.7, seed=941, width_bits=kw)
+        o = OracleTree(keys, W.rank_values(n, vw), 16, val_bits=vw)
+    tree = bt.BTree(keys, W.rank_values(n, vw), 16)
+    off = 1 if where == "misaligned" else 0
+
+    def buf(nbytes, pin):
+        return torch.full((nbytes + off,), 9, dtype=torch.uint8, pin_memory=pin)[off:]
+
+    raw = torch.from_numpy(q.view(np.uint8).reshape(-1).copy())
+    hq = buf(max(raw.numel(), nq * vw // 8), where not in ("pageable", "results"))
+    hq[: raw.numel()] = raw
+    hv = hq if where == "shared" else buf(nq * vw // 8, where not in ("pageable", "queries"))
+    hf = buf(nq, where not in ("pageable", "queries"))
+    ws, nb = tree.alloc_workspace(nq, host=True)
+    bt.bt_search_batch_host(tree.handle, hq, nq, hv, hf, ws, nb)
+    torch.cuda.synchronize()
+    ov, of = o.search(q)[:2]
+    got = hv[: nq * vw // 8].numpy().copy().view(np.uint64 if vw == 64 else np.uint32)
+    assert np.array_equal(got.astype(np.uint64), ov) and np.array_equal(hf.numpy(), of)
