@@ -133,8 +133,9 @@ typedef struct bt_info {
  * Beside the image, in an allocation of its own that bt_info does not count,
  * the device keeps a walk index: the keys and values once more in 64-byte
  * entries under 32-byte nodes, through which batches are searched as given
- * (see bt_search_opts.sort_bits).  It takes about 20 bytes per 64-bit key
- * and value (12 for 32-bit ones, 70 per 32-byte key) and is left out when
+ * (see bt_search_opts.sort_bits).  It takes about 17 bytes per 64-bit key
+ * and value (8.5 for 32-bit ones, 66 per 32-byte key), more where keys crowd
+ * (up to 20, 9 and 72), and is left out when
  * that is more than a quarter of the free device memory; searches are then
  * partitioned and descend the tree as bt_sort_bits says.
  *

@@ -83,15 +83,18 @@ struct PaperTree {
 // The walk index of a tree (walk.cuh), passed to kernels by value.
 constexpr int kWalkLevels = 12;
 struct WalkDev {
-    const unsigned char *top;      // segments' largest keys, a binary tree in breadth-first order
+    const unsigned char *top;      // separators of the segments, bin table, octave table
     const unsigned char *nodes;    // 32-byte nodes, level 0 (one node per segment) first
     const unsigned char *entries;  // 64-byte entries
     uint64_t off[kWalkLevels];     // byte offset of each level in nodes
     uint64_t n;                    // keys
+    uint64_t wmin, wmax;           // smallest and largest key (32-byte keys: word)
     uint64_t kmin32[4], kmax32[4]; // 32-byte keys: the smallest and largest key
     int p0;                        // 32-byte keys: bytes all keys share; the word walked follows them
     int levels;                    // levels of nodes
-    int top_bits;                  // depth of the binary tree (0: one segment, no top)
+    int coded;                     // of them coded, at the bottom (0, 1 or 2)
+    uint32_t segs, span;           // segments, entries per segment
+    uint32_t bin_off, oct_off;     // byte offsets of the two tables in top
     uint32_t top_bytes;
 };
 

@@ -509,7 +509,7 @@ extern "C" bt_status bt_build(const void *h_keys, const void *h_vals, uint64_t n
     d.split_off = kb == 32 ? static_cast<unsigned char *>(t->d_image) + split_off_offset : nullptr;
     d.split_R = reinterpret_cast<const uint16_t *>(static_cast<unsigned char *>(t->d_image) + split_R_offset);
     t->info.d_image = t->d_image;
-    e = walk_build(t, s);
+    e = walk_build(t, h_keys, s);
     if (e != cudaSuccess) {
         set_error_detail("walk index", e);
         bt_free(t);

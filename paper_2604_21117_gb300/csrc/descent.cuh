@@ -374,11 +374,11 @@ cudaError_t descend_synchronous(const DescendArgs &a, cudaStream_t s);
 cudaError_t descend_paper_layout(const DevTree &t, const PaperTree &p, const void *q, const uint32_t *qidx,
                                  const void *recs, uint64_t nq, void *out_v, uint8_t *out_f, cudaStream_t s);
 
-// Builds the walk index of a tree whose image is on the device, in an
-// allocation of its own.  Leaves the tree without one (and returns
+// Builds the walk index of a tree whose image is on the device (h_keys: the
+// sorted keys it was built from), in an allocation of its own.  Leaves the tree without one (and returns
 // cudaSuccess) when the index would take more than a quarter of the free
 // device memory, or the key count exceeds what its node numbers hold.
-cudaError_t walk_build(bt_tree *tree, cudaStream_t s);
+cudaError_t walk_build(bt_tree *tree, const void *h_keys, cudaStream_t s);
 // Search of a batch as given through the walk index; md: with a model of the
 // tree (integer keys).
 cudaError_t walk_search(const bt_tree *tree, const void *q, uint64_t nq, void *out_v, uint8_t *out_f, cudaStream_t s,

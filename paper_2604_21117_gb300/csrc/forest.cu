@@ -64,9 +64,9 @@ constexpr uint32_t kForestSmemList = 64;  // work lists up to this long are read
 constexpr uint32_t kForestPinMax = 98304;
 constexpr int kForestSmemMax = 200 * 1024;
 // Tops of a forest's trees in shared memory.  10,000 batches over trees of
-// 10^3, 10^5, 10^6 and 2 * 10^7 uint64 keys (146 KB of tops): 58.9 us with all
-// of them there, 71.7 with 96 KB (the largest tree's top through L1), 68.9
-// with none.
+// 10^3, 10^5, 10^6 and 2 * 10^7 uint64 keys, with tops searched by bisection
+// (146 KB): 58.9 us with all of them there, 71.7 with 96 KB (the largest
+// tree's top through L1), 68.9 with none.
 constexpr uint32_t kWalkTopBudget = 160 * 1024;
 
 __host__ __device__ inline uint32_t forest_desc_chunks(const bt_batch_desc &bd, uint32_t ntrees, uint64_t nq,
@@ -560,8 +560,8 @@ static std::vector<ForestWalk> walk_table(bt_forest *f)
         if (f->trees[i]->d_walk) tab[i].w = f->trees[i]->walk;
         tab[i].top_off = kNoTop;
         // in units of one probe of the top: a sector from the L2 costs about
-        // six, the entry two, the rest of a chunk's work about ten
-        tab[i].cost = 22u + static_cast<uint32_t>(tab[i].w.top_bits + 6 * tab[i].w.levels);
+        // six, the entry two, the top and the rest of a chunk's work about 16
+        tab[i].cost = 28u + static_cast<uint32_t>(6 * tab[i].w.levels);
     }
     std::sort(order.begin(), order.end(),
               [&](uint32_t a, uint32_t b) { return tab[a].w.top_bytes < tab[b].w.top_bytes; });

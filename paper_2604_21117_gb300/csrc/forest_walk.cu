@@ -218,11 +218,9 @@ __global__ void __launch_bounds__(kWalkForestThreads)
             V val = static_cast<V>(~static_cast<V>(0));
             bool hit = false;
             if (F.w.n) {
-                const uint32_t seg =
-                    F.top_off != kNoTop
-                        ? walk_segment<K>(reinterpret_cast<const K *>(smem + F.top_off), F.w.top_bits, now.key)
-                        : walk_segment_l1<K>(F.w.top, F.w.top_bits, now.key);
-                hit = walk_lookup<K, V>(F.w, walk_entry<K>(F.w, seg, now.key), now.key, val);
+                const unsigned char *top = F.top_off != kNoTop ? smem + F.top_off : F.w.top;
+                const uint32_t seg = walk_segment<K>(F.w, top, now.key);
+                hit = walk_lookup<K, V>(F.w, walk_entry<K>(F.w, top, seg, now.key), now.key, val);
             }
             if (now.valid) {
                 out_v[now.pos] = val;

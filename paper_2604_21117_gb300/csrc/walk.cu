@@ -4,6 +4,7 @@
 
 #include <cstdint>
 #include <cstring>
+#include <vector>
 
 #include "walk.cuh"
 
@@ -71,24 +72,56 @@ __global__ void k_walk_nodes(LeafView lv, uint64_t nodes, uint64_t span, uint64_
     }
 }
 
-// The binary tree over the segments' largest keys (all but the last
-// segment's): position k at depth d holds the separator of sorted rank
-// ((2 (k - 2^d) + 1) << (bits - 1 - d)) - 1.
+// The words that bound the keys of coded node `root`, which spans `span`
+// entries: (lo, hi].
 template <typename K>
-__global__ void k_walk_top(LeafView lv, int bits, uint64_t span, uint64_t E, uint32_t G, int p0,
-                           typename WalkWord<K>::type *__restrict__ out)
+__device__ __forceinline__ void root_bounds(const LeafView &lv, uint64_t root, uint64_t span, uint64_t n, uint32_t G,
+                                            int p0, typename WalkWord<K>::type &lo, typename WalkWord<K>::type &hi)
+{
+    const uint64_t first = root * span * G, end = first + span * G;
+    lo = walk_word<K>(lv, first ? first - 1 : 0, p0);
+    hi = walk_word<K>(lv, (end < n ? end : n) - 1, p0);
+}
+
+// One thread per code of a coded level whose nodes' children span `span`
+// entries, under roots of `root_span` entries.
+template <typename K>
+__global__ void k_walk_codes(LeafView lv, uint64_t nodes, uint64_t span, uint64_t root_span, uint64_t n, uint64_t E,
+                             uint32_t G, int p0, uint16_t *__restrict__ out)
 {
     using W = typename WalkWord<K>::type;
-    const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= (1u << bits)) return;
-    W v = static_cast<W>(~static_cast<W>(0));
-    if (k > 0) {
-        const int d = 31 - __clz(k);
-        const uint64_t rank = (static_cast<uint64_t>(2u * (k - (1u << d)) + 1u) << (bits - 1 - d)) - 1;
-        const uint64_t end = (rank + 1) * span;
-        if (end < E) v = walk_word<K>(lv, end * G - 1, p0);
+    constexpr uint32_t SEP = kCodeFan - 1;
+    for (uint64_t i = blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x; i < nodes * SEP;
+         i += static_cast<uint64_t>(gridDim.x) * blockDim.x) {
+        const uint64_t end = (i / SEP * kCodeFan + i % SEP + 1) * span;  // entries up to this child's last
+        uint32_t code = 0xFFFFu;
+        if (end < E) {
+            W lo, hi;
+            root_bounds<K>(lv, (end - 1) / root_span, root_span, n, G, p0, lo, hi);
+            code = walk_code<W>(walk_word<K>(lv, end * G - 1, p0), lo, hi);
+        }
+        out[i] = static_cast<uint16_t>(code);
     }
-    out[k] = v;
+}
+
+// Neighbouring entries under one root whose largest keys' codes tie.
+template <typename K>
+__global__ void k_walk_ties(LeafView lv, uint64_t root_span, uint64_t n, uint64_t E, uint32_t G, int p0,
+                            unsigned long long *__restrict__ ties)
+{
+    using W = typename WalkWord<K>::type;
+    unsigned long long mine = 0;
+    for (uint64_t i = blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x; i + 1 < E;
+         i += static_cast<uint64_t>(gridDim.x) * blockDim.x) {
+        if (i / root_span != (i + 1) / root_span) continue;
+        W lo, hi;
+        root_bounds<K>(lv, i / root_span, root_span, n, G, p0, lo, hi);
+        const uint64_t next = (i + 2) * G;
+        if (walk_code<W>(walk_word<K>(lv, (i + 1) * G - 1, p0), lo, hi) ==
+            walk_code<W>(walk_word<K>(lv, (next < n ? next : n) - 1, p0), lo, hi))
+            ++mine;
+    }
+    if (mine) atomicAdd(ties, mine);
 }
 
 static unsigned fill_grid(uint64_t items)
@@ -98,21 +131,52 @@ static unsigned fill_grid(uint64_t items)
 }
 
 template <typename K>
-static cudaError_t build_levels(WalkDev &w, const LeafView &lv, uint64_t E, uint32_t G, const uint64_t *count,
-                                unsigned char *top, unsigned char *nodes, cudaStream_t s)
+static cudaError_t build_levels(const WalkDev &w, const LeafView &lv, uint64_t E, uint32_t G, const uint64_t *count,
+                                unsigned char *nodes, cudaStream_t s)
 {
     using W = typename WalkWord<K>::type;
     constexpr uint64_t F = 32 / sizeof(W) + 1;
-    uint64_t span = 1;
+    uint64_t span = 1, root_span = 1;
+    for (int l = 0; l < w.coded; ++l) root_span *= kCodeFan;
     for (int l = w.levels - 1; l >= 0; --l) {
-        k_walk_nodes<K><<<fill_grid(count[l] * (F - 1)), 256, 0, s>>>(lv, count[l], span, E, G, w.p0,
-                                                                     reinterpret_cast<W *>(nodes + w.off[l]));
-        span *= F;
+        if (l >= w.levels - w.coded) {
+            k_walk_codes<K><<<fill_grid(count[l] * (kCodeFan - 1)), 256, 0, s>>>(
+                lv, count[l], span, root_span, w.n, E, G, w.p0, reinterpret_cast<uint16_t *>(nodes + w.off[l]));
+            span *= kCodeFan;
+        } else {
+            k_walk_nodes<K><<<fill_grid(count[l] * (F - 1)), 256, 0, s>>>(lv, count[l], span, E, G, w.p0,
+                                                                         reinterpret_cast<W *>(nodes + w.off[l]));
+            span *= F;
+        }
     }
-    if (w.top_bits)
-        k_walk_top<K><<<(1u << w.top_bits) / 256 + 1, 256, 0, s>>>(lv, w.top_bits, span, E, G, w.p0,
-                                                                  reinterpret_cast<W *>(top));
     return cudaGetLastError();
+}
+
+// Whether codes of `coded` levels would tie for more than one entry in 256.
+// Every query of a tied run goes on from the run's first entry: 2^20 queries
+// over 2^23 uniform keys, with one key in 1000 / 200 / 100 / 50 of them in
+// dense runs of 40 (a tenth, half, one and two percent of the entries tie):
+// 30.1 / 31.7 / 33.3 / 36.0 us through codes, 31.9 through full words at any
+// share (27.9 and 31.9 without runs).
+template <typename K>
+static cudaError_t codes_tie(const LeafView &lv, int coded, uint64_t n, uint64_t E, uint32_t G, int p0, bool *tie,
+                             cudaStream_t s)
+{
+    uint64_t root_span = 1;
+    for (int l = 0; l < coded; ++l) root_span *= kCodeFan;
+    unsigned long long *d = nullptr, h = 0;
+    cudaError_t e = cudaMalloc(&d, sizeof(h));
+    if (e != cudaSuccess) return e;
+    e = cudaMemsetAsync(d, 0, sizeof(h), s);
+    if (e == cudaSuccess) {
+        k_walk_ties<K><<<fill_grid(E), 256, 0, s>>>(lv, root_span, n, E, G, p0, d);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&h, d, sizeof(h), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    cudaFree(d);
+    *tie = h > E / 256;
+    return e;
 }
 
 template <typename K, typename V>
@@ -123,12 +187,60 @@ static cudaError_t build_entries(const LeafView &lv, uint64_t n, uint64_t E, uin
     return cudaGetLastError();
 }
 
-cudaError_t walk_build(bt_tree *t, cudaStream_t s)
+// The word of the key of rank i in the caller's array.
+static uint64_t host_word(const void *h_keys, uint64_t i, int kb, int p0)
+{
+    if (kb == 8) return static_cast<const uint64_t *>(h_keys)[i];
+    if (kb == 4) return static_cast<const uint32_t *>(h_keys)[i];
+    const unsigned char *b = static_cast<const unsigned char *>(h_keys) + i * 32 + p0;
+    uint64_t v = 0;
+    for (int j = 0; j < 8; ++j) v = v << 8 | b[j];
+    return v;
+}
+
+// The top: separators (the last one the largest word), bins, octaves.
+template <typename W>
+static std::vector<unsigned char> build_top(WalkDev &w, const std::vector<uint64_t> &sep)
+{
+    uint32_t held[64] = {};
+    std::vector<uint32_t> oct(sep.size());
+    std::vector<uint64_t> x(sep.size());
+    for (size_t i = 0; i + 1 < sep.size(); ++i) {
+        oct[i] = walk_octave<W>(w, static_cast<W>(sep[i]), x[i]);
+        ++held[oct[i]];
+    }
+    WalkOctave table[64];
+    uint32_t bins = 0;
+    for (int o = 0; o < 64; ++o) {
+        int bits = 0;
+        while (bits < o && (2u << bits) <= held[o]) ++bits;
+        table[o] = WalkOctave{bins, static_cast<uint32_t>(o - bits)};
+        bins += 1u << bits;
+    }
+    w.bin_off = static_cast<uint32_t>((sep.size() * sizeof(W) + 15) / 16 * 16);
+    w.oct_off = static_cast<uint32_t>((w.bin_off + (bins + 1) * 2 + 15) / 16 * 16);
+    w.top_bytes = w.oct_off + static_cast<uint32_t>(sizeof(table));
+    std::vector<unsigned char> top(w.top_bytes, 0);
+    W *s = reinterpret_cast<W *>(top.data());
+    uint16_t *first = reinterpret_cast<uint16_t *>(top.data() + w.bin_off);
+    size_t at = 0;
+    for (size_t i = 0; i < sep.size(); ++i) {
+        s[i] = static_cast<W>(sep[i]);
+        if (i + 1 == sep.size()) break;
+        const uint32_t bin = table[oct[i]].base + static_cast<uint32_t>(x[i] >> table[oct[i]].shift);
+        while (at <= bin) first[at++] = static_cast<uint16_t>(i);
+    }
+    while (at <= bins) first[at++] = static_cast<uint16_t>(sep.size() - 1);
+    memcpy(top.data() + w.oct_off, table, sizeof(table));
+    return top;
+}
+
+cudaError_t walk_build(bt_tree *t, const void *h_keys, cudaStream_t s)
 {
     const DevTree &d = t->dev;
     const uint64_t n = t->info.n;
     if (n == 0) return cudaSuccess;
-    const int kb = d.key_bytes, vb = d.val_bytes, wb = kb > 8 ? 8 : kb;
+    const int kb = d.key_bytes, vb = d.val_bytes;
     const uint32_t G = walk_group(kb, vb);
     const uint64_t F = walk_fan(kb), E = (n + G - 1) / G;
     if (E >= (1ull << 32)) return cudaSuccess;  // node and entry numbers are 32-bit
@@ -138,22 +250,53 @@ cudaError_t walk_build(bt_tree *t, cudaStream_t s)
     w.p0 = d.split_p0;
     memcpy(w.kmin32, d.kmin32, sizeof(w.kmin32));
     memcpy(w.kmax32, d.kmax32, sizeof(w.kmax32));
-    // as few levels of nodes as leave at most 2^walk_top_bits segments
-    uint64_t segs = E, count[kWalkLevels];
-    while (segs > (1ull << walk_top_bits(kb))) {
+    w.wmin = host_word(h_keys, 0, kb, w.p0);
+    w.wmax = host_word(h_keys, n - 1, kb, w.p0);
+    const int leaf = d.height - 1;
+    const LeafView lv{d.keys[leaf], d.vals, d.cbase[leaf], d.crem[leaf], static_cast<uint32_t>(d.m)};
+    cudaError_t e = cudaSuccess;
+    // coded levels: one where it leaves at most kWalkSegs segments, else two;
+    // none where codes tie; then levels of full words down to kWalkMaxSegs
+    // (without codes kWalkMaxSegs / 2, as those trees' tops measured best)
+    uint64_t segs = E, span = 1, count[kWalkLevels];
+    if (E > kWalkSegs) {
+        w.coded = (E + kCodeFan - 1) / kCodeFan <= kWalkSegs ? 1 : 2;
+        bool tie = false;
+        e = kb == 32 ? codes_tie<Key32>(lv, w.coded, n, E, G, w.p0, &tie, s)
+            : kb == 8 ? codes_tie<uint64_t>(lv, w.coded, n, E, G, w.p0, &tie, s)
+                      : codes_tie<uint32_t>(lv, w.coded, n, E, G, w.p0, &tie, s);
+        if (e == cudaErrorMemoryAllocation) {
+            cudaGetLastError();  // no room for an index then
+            return cudaSuccess;
+        }
+        if (e != cudaSuccess) return e;
+        if (tie) w.coded = 0;
+    }
+    for (int l = 0; l < w.coded; ++l) {
+        segs = (segs + kCodeFan - 1) / kCodeFan;
+        span *= kCodeFan;
+    }
+    w.levels = w.coded;
+    while (segs > (w.coded ? kWalkMaxSegs : kWalkMaxSegs / 2)) {
         segs = (segs + F - 1) / F;
+        span *= F;
         ++w.levels;
     }
     uint64_t c = E;
     for (int l = w.levels - 1; l >= 0; --l) {
-        c = (c + F - 1) / F;
+        const uint64_t fan = l >= w.levels - w.coded ? kCodeFan : F;
+        c = (c + fan - 1) / fan;
         count[l] = c;
     }
-    if (segs > 1) {
-        w.top_bits = 2;  // whole 16-byte pieces for the bulk copy
-        while ((1ull << w.top_bits) < segs) ++w.top_bits;
-        w.top_bytes = static_cast<uint32_t>(wb) << w.top_bits;
+    w.segs = static_cast<uint32_t>(segs);
+    w.span = static_cast<uint32_t>(span);
+    std::vector<uint64_t> sep(segs);
+    for (uint64_t i = 0; i < segs; ++i) {
+        const uint64_t end = (i + 1) * span * G;
+        sep[i] = host_word(h_keys, (end < n ? end : n) - 1, kb, w.p0);
     }
+    std::vector<unsigned char> top;
+    if (segs > 1) top = kb == 4 ? build_top<uint32_t>(w, sep) : build_top<uint64_t>(w, sep);
     uint64_t bytes = (static_cast<uint64_t>(w.top_bytes) + 255) & ~255ull;
     const uint64_t node_off = bytes;
     for (int l = 0; l < w.levels; ++l) {
@@ -164,7 +307,7 @@ cudaError_t walk_build(bt_tree *t, cudaStream_t s)
     const uint64_t ent_off = bytes;
     bytes += E * 64;
     size_t free_b = 0, total_b = 0;
-    cudaError_t e = cudaMemGetInfo(&free_b, &total_b);
+    e = cudaMemGetInfo(&free_b, &total_b);
     if (e != cudaSuccess) return e;
     if (bytes > free_b / 4) return cudaSuccess;
     e = cudaMalloc(&t->d_walk, bytes);
@@ -178,21 +321,21 @@ cudaError_t walk_build(bt_tree *t, cudaStream_t s)
     w.top = base;
     w.nodes = base + node_off;
     w.entries = base + ent_off;
-    const int leaf = d.height - 1;
-    const LeafView lv{d.keys[leaf], d.vals, d.cbase[leaf], d.crem[leaf], static_cast<uint32_t>(d.m)};
     unsigned char *nodes = base + node_off, *ent = base + ent_off;
+    if (w.top_bytes) e = cudaMemcpyAsync(base, top.data(), top.size(), cudaMemcpyHostToDevice, s);
+    if (e != cudaSuccess) return e;
     if (kb == 32) {
-        e = build_levels<Key32>(w, lv, E, G, count, base, nodes, s);
+        e = build_levels<Key32>(w, lv, E, G, count, nodes, s);
         if (e == cudaSuccess)
             e = vb == 8 ? build_entries<Key32, uint64_t>(lv, n, E, G, ent, s)
                         : build_entries<Key32, uint32_t>(lv, n, E, G, ent, s);
     } else if (kb == 8) {
-        e = build_levels<uint64_t>(w, lv, E, G, count, base, nodes, s);
+        e = build_levels<uint64_t>(w, lv, E, G, count, nodes, s);
         if (e == cudaSuccess)
             e = vb == 8 ? build_entries<uint64_t, uint64_t>(lv, n, E, G, ent, s)
                         : build_entries<uint64_t, uint32_t>(lv, n, E, G, ent, s);
     } else {
-        e = build_levels<uint32_t>(w, lv, E, G, count, base, nodes, s);
+        e = build_levels<uint32_t>(w, lv, E, G, count, nodes, s);
         if (e == cudaSuccess)
             e = vb == 8 ? build_entries<uint32_t, uint64_t>(lv, n, E, G, ent, s)
                         : build_entries<uint32_t, uint32_t>(lv, n, E, G, ent, s);
@@ -214,7 +357,6 @@ constexpr int walk_threads()
 struct WalkModel {
     ModelDev md;
     uint64_t leaf_base, leaf_rem;  // keys per leaf, leaves with one more
-    uint32_t span;                 // entries per segment
 };
 
 // One query per lane, one block per SM; every block takes a contiguous run
@@ -223,15 +365,19 @@ struct WalkModel {
 // copied once per block by one bulk copy, before the wait for the previous
 // kernel of the stream.
 //
-// What bounds it: divergent sectors.  A warp's 32-lane read of one sector
-// per lane occupies an SM for 34 cycles when it comes from the L2 and 20
-// when it hits L1; an 8-byte probe of the top in shared memory for 6 (5-ary
-// nodes in shared memory: 30 per level, so the top is binary).  Over 2^24
-// uint64 keys a query is 13 probes, four nodes and an entry of two sectors,
-// about 290 cycles per warp, 30 us for 2^20 queries; measured 41.1 us with
-// three trees in turn (38.7 for one), against 92.4 us for the partition and
-// the level-wise descent.  1024 threads on one SM: with two blocks of 768 or
-// 512 the two copies of the top take the L1 the nodes want (42-67 us).
+// What bounds it: divergent reads.  A warp's read of one sector per lane
+// occupies an SM for 34 cycles when it comes from the L2 and 20 when it hits
+// L1, whatever part of the sector is used; a probe of the top in shared
+// memory for 6; and 2^20 reads of random entries of 64 bytes take 18 us from
+// memory by themselves.  Over 2^24 uint64 keys a query is about six probes,
+// two coded nodes, an entry's keys and one value: 33.6 us for 2^20 queries
+// with three trees in turn (31.5 for one).  Before the walk, the partition
+// and the level-wise descent: 92.4 us; with four nodes of full words under a
+// top searched by bisection (13 probes): 41.6; with the top's tables 41.2.
+// For 32-byte keys (2^20 keys) 113, 38.6, 36.9, now 31.4 us.
+// 1024 threads on one SM: two blocks (of 1024, 768 or 512) hold two copies
+// of the top and gain nothing from the additional warps (2^20 queries over
+// 2^24 keys, full-word nodes: 42.3, 43.5 and 51.4 us against 40.4).
 // The kernel does not trigger the launch of its successor: blocks started
 // early pair up on the SMs that drain first, and the batch then waits for
 // those (300,007 uint32 queries: 15.0 us with the trigger, 8.6 without).
@@ -287,22 +433,26 @@ __global__ void __launch_bounds__(walk_threads<MODEL>())
         } else {
             word = key;
         }
-        const W *top = reinterpret_cast<const W *>(smem);
         uint32_t seg;
         if constexpr (MODEL == kModelNone) {
-            seg = walk_segment<W>(top, w.top_bits, word);
+            seg = walk_segment<W>(w, smem, word);
         } else {
             constexpr uint32_t G = walk_group(sizeof(K), sizeof(V));
+            const W *sep = reinterpret_cast<const W *>(smem);
             uint32_t lo, hi;
             model_window<MODEL>(m.md, mv, static_cast<uint64_t>(key), lo, hi);
             // first key of leaf lo, last key of leaf hi, as entries, as segments
             const uint64_t r0 = lo * m.leaf_base + (lo < m.leaf_rem ? lo : m.leaf_rem);
             const uint64_t r1 = (hi + 1ull) * m.leaf_base + (hi + 1ull < m.leaf_rem ? hi + 1ull : m.leaf_rem) - 1;
-            seg = walk_segment_in<W>(top, w.top_bits, static_cast<uint32_t>(r0 / G) / m.span,
-                                     static_cast<uint32_t>(r1 / G) / m.span, word);
+            const uint32_t s0 = static_cast<uint32_t>(r0 / G) / w.span, s1 = static_cast<uint32_t>(r1 / G) / w.span;
+            // proven by the separators on both sides, else the whole top searched
+            if ((s0 == 0 || sep[s0 - 1] < word) && (s1 + 1 >= w.segs || !(sep[s1] < word)))
+                seg = walk_segment_in<W>(sep, s0, s1, word);
+            else
+                seg = walk_segment<W>(w, smem, word);
         }
         V val;
-        bool hit = walk_lookup<K, V>(w, walk_entry<W>(w, seg, word), key, val);
+        bool hit = walk_lookup<K, V>(w, walk_entry<W>(w, smem, seg, word), key, val);
         if (!in) {
             hit = false;
             val = static_cast<V>(~static_cast<V>(0));
@@ -321,7 +471,7 @@ static cudaError_t walk_launch(const bt_tree *t, const ModelDev *md, const void 
 {
     auto kern = k_walk<K, V, MODEL>;
     const WalkDev &w = t->walk;
-    constexpr int kMaxTop = static_cast<int>(sizeof(typename WalkWord<K>::type)) << walk_top_bits(sizeof(K));
+    constexpr int kMaxTop = walk_max_top(sizeof(K));
     constexpr int kMaxModel = MODEL == kModelNone ? 0 : static_cast<int>(kModelSmemSegments) * 20;
     int sms = 0;
     cudaError_t e = dev_sm_count(&sms);
@@ -334,8 +484,6 @@ static cudaError_t walk_launch(const bt_tree *t, const ModelDev *md, const void 
         m.md = *md;
         m.leaf_base = t->dev.cbase[leaf];
         m.leaf_rem = t->dev.crem[leaf];
-        m.span = 1;
-        for (int l = 0; l < w.levels; ++l) m.span *= walk_fan(static_cast<int>(sizeof(K)));
     }
     // one block per SM with as many warps as its share of the chunks
     constexpr uint64_t kWarps = walk_threads<MODEL>() / 32;

@@ -35,12 +35,12 @@ def _same(tree, o, q):
         assert np.array_equal(f.cpu().numpy(), of)
 
 
-# entries hold 32 / max(widths) keys, the top 2^13 segments (2^14 for 32-bit
-# keys), a node 5 children (9 for 32-bit keys)
+# entries hold 32 / max(widths) keys; up to 2^12 entries the top alone, then
+# one coded level of 17 children up to 2^12 segments, then two
 @pytest.mark.parametrize("kw,vw,n", [
-    (64, 64, 1), (64, 64, 4), (64, 64, 5), (64, 64, 4 * 8192), (64, 64, 4 * 8192 + 1), (64, 64, 4 * 5 * 8192),
-    (64, 64, 4 * 5 * 8192 + 1), (64, 64, 4 * 25 * 8192 + 3), (64, 32, 4 * 8192 + 2), (32, 64, 4 * 16384 + 1),
-    (32, 32, 7), (32, 32, 8 * 16384), (32, 32, 8 * 16384 + 1), (32, 32, 8 * 9 * 16384 + 5)])
+    (64, 64, 1), (64, 64, 4), (64, 64, 5), (64, 64, 4 * 4096), (64, 64, 4 * 4096 + 1), (64, 64, 4 * 17 * 4096),
+    (64, 64, 4 * 17 * 4096 + 1), (64, 64, 4 * 289 * 700 + 3), (64, 32, 4 * 4096 + 2), (32, 64, 4 * 4096 + 1),
+    (32, 32, 7), (32, 32, 8 * 4096), (32, 32, 8 * 4096 + 1), (32, 32, 8 * 17 * 4096), (32, 32, 8 * 17 * 4096 + 5)])
 @pytest.mark.parametrize("nq", [1, 33, 152 * 1024 + 33])
 def test_index_shape_boundaries(bt, kw, vw, n, nq):
     keys = W.uniform_keys(n, kw, seed=900 + n)
@@ -61,7 +61,40 @@ def test_all_ones_key_stored_and_not(bt):
         _same(tree, o, np.array([top, top - 1, 0, 1, 4, 5], np.uint64))
 
 
-@pytest.mark.parametrize("n", [1, 2, 8192, 8193, 5 * 8192 + 1])
+def _crowded(kind, kw, n):
+    """Keys whose distances inside a few hundred entries differ too much for
+    16-bit codes: everywhere ("runs": nodes of full words, several levels of
+    them), in one key of 300 ("some": codes that tie here and there), at both
+    ends, and all keys consecutive (codes are exact)."""
+    g = W.rng(915)
+    i = np.arange(n, dtype=np.uint64)
+    if kind == "runs":
+        return (i // 100 << np.uint64(kw // 2)) | i % 100 if kw == 64 else (i // 20 << np.uint64(11)) | i % 20
+    if kind == "dense":
+        return i + np.uint64(12345)
+    far = W.uniform_keys(n - n // 300, kw, seed=916).astype(np.uint64)
+    if kind == "some":
+        starts = g.choice(far, size=n // 300 // 40 + 1)
+        near = (starts[:, None] + np.arange(1, 41, dtype=np.uint64)).ravel()
+    else:
+        near = np.concatenate([i[: n // 100], np.uint64(2**kw - 1) - i[: n // 100]])
+    return np.unique(np.concatenate([far, near]))
+
+
+@pytest.mark.parametrize("kind", ["runs", "some", "ends", "dense"])
+@pytest.mark.parametrize("kw,n", [(64, 100_000), (64, 1_500_000), (32, 1_500_000)])
+def test_keys_that_crowd(bt, kind, kw, n):
+    keys = _crowded(kind, kw, n).astype(W.key_dtype(kw))
+    vals = W.rank_values(keys.size, 64)
+    tree = bt.BTree(keys, vals, 32)
+    o = OracleTree(keys, vals, 32)
+    g = W.rng(917)
+    near = keys[g.integers(0, keys.size, size=30_000)] + g.integers(0, 3, size=30_000).astype(keys.dtype)
+    _same(tree, o, np.concatenate([W.make_queries(keys, 30_001, 0.8, seed=918, width_bits=kw), near, keys[:3],
+                                   keys[-3:]]))
+
+
+@pytest.mark.parametrize("n", [1, 2, 4096, 4097, 17 * 4096 + 1])
 @pytest.mark.parametrize("tie", [0, 7, 5000])
 def test_byte_keys_with_tied_words(bt, n, tie):
     """Runs of `tie` keys that share the 8 bytes the index walks and differ
