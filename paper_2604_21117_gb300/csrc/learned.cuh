@@ -79,12 +79,30 @@ __device__ __forceinline__ int pl_segment(const uint64_t *b, uint32_t S, uint64_
     return lo;
 }
 
+// fp32(fp64(d)), the two roundings of the models' definition, by integer
+// steps (the fp64 unit takes 16 cycles per warp instruction): d is rounded to
+// 53 bits, ties to even, where it has more, and the result to 24 by the
+// conversion.
+__device__ __forceinline__ float float_of_double(uint64_t d)
+{
+    const int drop = 11 - __clzll(static_cast<long long>(d));  // bits beyond 53
+    if (drop > 0) {
+        const uint64_t half = 1ull << (drop - 1), rest = d & ((1ull << drop) - 1);
+        uint64_t t = d >> drop;
+        t += (rest > half || (rest == half && (t & 1u))) ? 1u : 0u;
+        // t may have become 2^53; t << drop may be 2^64, which the shift below drops
+        if (t >> (64 - drop)) return 18446744073709551616.0f;
+        d = t << drop;
+    }
+    return __ull2float_rn(d);
+}
+
 __device__ __forceinline__ float pl_predict(const uint64_t *b, const float *inv_w, const float *slope,
                                             const float *icpt, uint32_t S, uint64_t q)
 {
     const int s = pl_segment(b, S, q);
     const uint64_t diff = q >= b[s] ? q - b[s] : 0ull;
-    const float x = __fmul_rn(__double2float_rn(__ull2double_rn(diff)), inv_w[s]);
+    const float x = __fmul_rn(float_of_double(diff), inv_w[s]);
     return __fadd_rn(__fmul_rn(slope[s], x), icpt[s]);
 }
 
@@ -94,7 +112,7 @@ __device__ __forceinline__ float mlp_x_rank(const uint64_t *b, const float *inv_
 {
     const int s = pl_segment(b, kMlpStage1, q);
     const uint64_t diff = q >= b[s] ? q - b[s] : 0ull;
-    const float u = fminf(__fmul_rn(__double2float_rn(__ull2double_rn(diff)), inv_w[s]), 1.0f);
+    const float u = fminf(__fmul_rn(float_of_double(diff), inv_w[s]), 1.0f);
     return __fmul_rn(__fadd_rn(static_cast<float>(s), u), 1.0f / static_cast<float>(kMlpStage1));
 }
 

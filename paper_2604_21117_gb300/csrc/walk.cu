@@ -359,6 +359,41 @@ struct WalkModel {
     uint64_t leaf_base, leaf_rem;  // keys per leaf, leaves with one more
 };
 
+// The model's parameters in shared memory behind the top, each array rounded
+// up to whole 16-byte pieces (the model's allocation pads them).
+__host__ __device__ inline uint32_t walk_model_bytes(const ModelDev &m)
+{
+    if (m.kind == kModelPL)
+        return m.segments <= kModelSmemSegments ? (m.segments * 8u + 15u) / 16u * 16u + 3u * ((m.segments * 4u + 15u) / 16u * 16u) : 0u;
+    if (m.kind == kModelMLP) return kMlpStage1 * 12u + (kMlpParams * 4u + 15u) / 16u * 16u;
+    return 0u;
+}
+
+// Where the parameters are, and (one thread, `copy`) their bulk copies.
+template <int MODEL>
+__device__ __forceinline__ ModelView walk_model(const ModelDev &md, unsigned char *msm, uint64_t *bar, bool copy)
+{
+    ModelView v{md.b, md.inv_w, md.slope, md.icpt, md.mlp};
+    if (walk_model_bytes(md) == 0) return v;
+    auto put = [&](const void *src, uint32_t bytes) {
+        const uint32_t padded = (bytes + 15u) / 16u * 16u;
+        unsigned char *dst = msm;
+        if (copy) bulk_g2s(dst, src, padded, bar);
+        msm += padded;
+        return dst;
+    };
+    const uint32_t S = MODEL == kModelPL ? md.segments : kMlpStage1;
+    v.b = reinterpret_cast<const uint64_t *>(put(md.b, S * 8u));
+    v.inv_w = reinterpret_cast<const float *>(put(md.inv_w, S * 4u));
+    if constexpr (MODEL == kModelPL) {
+        v.slope = reinterpret_cast<const float *>(put(md.slope, S * 4u));
+        v.icpt = reinterpret_cast<const float *>(put(md.icpt, S * 4u));
+    } else {
+        v.mlp = reinterpret_cast<const float *>(put(md.mlp, kMlpParams * 4u));
+    }
+    return v;
+}
+
 // One query per lane, one block per SM; every block takes a contiguous run
 // of 32-query chunks of the batch, its warps chunk by chunk in turn, the
 // next chunk's queries loaded while the present one walks.  The top is
@@ -396,11 +431,11 @@ __global__ void __launch_bounds__(walk_threads<MODEL>())
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     if (threadIdx.x == 0) {
         mbar_init(&bar);
-        mbar_arrive_expect_tx(&bar, w.top_bytes);
+        mbar_arrive_expect_tx(&bar, w.top_bytes + (MODEL == kModelNone ? 0u : walk_model_bytes(m.md)));
         if (w.top_bytes) bulk_g2s(smem, w.top, w.top_bytes, &bar);
     }
     ModelView mv{};
-    if constexpr (MODEL != kModelNone) mv = model_to_smem<MODEL>(m.md, smem + w.top_bytes);
+    if constexpr (MODEL != kModelNone) mv = walk_model<MODEL>(m.md, smem + w.top_bytes, &bar, threadIdx.x == 0);
     pdl_wait();
     const uint32_t chunks = (nq + 31) / 32;
     const uint32_t c1 = static_cast<uint32_t>(static_cast<uint64_t>(chunks) * (blockIdx.x + 1) / gridDim.x);
@@ -412,7 +447,7 @@ __global__ void __launch_bounds__(walk_threads<MODEL>())
     };
     K next = KeyOps<K>::ones();
     if (c < c1) next = load(c);
-    __syncthreads();  // the barrier is initialised, the model copied
+    __syncthreads();  // the barrier is initialised
     if (!mbar_wait_warp(&bar, 0, wait_polls)) {
         mbar_give_up(&bar, 0, static_cast<int>(lane));
         return;
@@ -472,7 +507,7 @@ static cudaError_t walk_launch(const bt_tree *t, const ModelDev *md, const void 
     auto kern = k_walk<K, V, MODEL>;
     const WalkDev &w = t->walk;
     constexpr int kMaxTop = walk_max_top(sizeof(K));
-    constexpr int kMaxModel = MODEL == kModelNone ? 0 : static_cast<int>(kModelSmemSegments) * 20;
+    constexpr int kMaxModel = MODEL == kModelNone ? 0 : static_cast<int>(kModelSmemSegments) * 20 + 64;
     int sms = 0;
     cudaError_t e = dev_sm_count(&sms);
     if (e == cudaSuccess) e = ensure_dyn_smem(reinterpret_cast<const void *>(kern), kMaxTop + kMaxModel);
@@ -495,7 +530,7 @@ static cudaError_t walk_launch(const bt_tree *t, const ModelDev *md, const void 
     memset(&cfg, 0, sizeof(cfg));
     cfg.gridDim = dim3(static_cast<unsigned>(grid));
     cfg.blockDim = dim3(static_cast<unsigned>(warps * 32));
-    cfg.dynamicSmemBytes = w.top_bytes + (MODEL == kModelNone ? 0u : model_smem_bytes(m.md));
+    cfg.dynamicSmemBytes = w.top_bytes + (MODEL == kModelNone ? 0u : walk_model_bytes(m.md));
     cfg.stream = s;
     cudaLaunchAttribute attr;
     memset(&attr, 0, sizeof(attr));
@@ -508,7 +543,7 @@ static cudaError_t walk_launch(const bt_tree *t, const ModelDev *md, const void 
 }
 
 template <typename K, typename V>
-static cudaError_t walk_model(const bt_tree *t, const ModelDev *md, const void *q, uint64_t nq, void *out_v,
+static cudaError_t walk_any(const bt_tree *t, const ModelDev *md, const void *q, uint64_t nq, void *out_v,
                               uint8_t *out_f, cudaStream_t s)
 {
     if constexpr (sizeof(K) <= 8) {
@@ -524,13 +559,13 @@ cudaError_t walk_search(const bt_tree *t, const void *q, uint64_t nq, void *out_
     const int kb = t->dev.key_bytes;
     const bool v8 = t->dev.val_bytes == 8;
     if (kb == 32)
-        return v8 ? walk_model<Key32, uint64_t>(t, md, q, nq, out_v, out_f, s)
-                  : walk_model<Key32, uint32_t>(t, md, q, nq, out_v, out_f, s);
+        return v8 ? walk_any<Key32, uint64_t>(t, md, q, nq, out_v, out_f, s)
+                  : walk_any<Key32, uint32_t>(t, md, q, nq, out_v, out_f, s);
     if (kb == 8)
-        return v8 ? walk_model<uint64_t, uint64_t>(t, md, q, nq, out_v, out_f, s)
-                  : walk_model<uint64_t, uint32_t>(t, md, q, nq, out_v, out_f, s);
-    return v8 ? walk_model<uint32_t, uint64_t>(t, md, q, nq, out_v, out_f, s)
-              : walk_model<uint32_t, uint32_t>(t, md, q, nq, out_v, out_f, s);
+        return v8 ? walk_any<uint64_t, uint64_t>(t, md, q, nq, out_v, out_f, s)
+                  : walk_any<uint64_t, uint32_t>(t, md, q, nq, out_v, out_f, s);
+    return v8 ? walk_any<uint32_t, uint64_t>(t, md, q, nq, out_v, out_f, s)
+              : walk_any<uint32_t, uint32_t>(t, md, q, nq, out_v, out_f, s);
 }
 
 cudaError_t take_wait_counters_walk(unsigned *timeouts, unsigned *pending)
