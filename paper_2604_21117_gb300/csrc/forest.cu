@@ -32,6 +32,7 @@
 #include "bt_internal.h"
 #include "descent.cuh"
 #include "forest.h"
+#include "walk.cuh"
 
 struct bt_forest {
     btgb::ForestTree *d_tab;
@@ -48,7 +49,7 @@ struct bt_forest {
     uint32_t stage_bytes;  // per warp, 0 when no tree is staged
     btgb::ForestWalk *d_walk;  // table of the walk kernel
     bool walk;             // work lists go to the walk kernel (every tree has a walk index or is empty, no
-                           // model, no tree staged per warp)
+                           // model, no tree staged per warp, a table that fits)
     uint32_t walk_top;     // bytes of the tops it copies to shared memory
     int model_set;         // kModelNone (no model), kModelPL (PL models only), kModelMLP (any model)
 };
@@ -543,7 +544,7 @@ static void forest_table(bt_forest *f)
         if (k == kModelPL && f->model_set == kModelNone) f->model_set = kModelPL;
     }
     f->stage_bytes = any_staged ? static_cast<uint32_t>(kForestStageBytes) : 0u;
-    f->walk = !any_staged && f->model_set == kModelNone;
+    f->walk = !any_staged && f->model_set == kModelNone && n <= kForestWalkTrees;
     for (uint32_t i = 0; i < n; ++i)
         if (f->trees[i]->dev.height > 0 && !f->trees[i]->d_walk) f->walk = false;
 }
@@ -559,9 +560,14 @@ static std::vector<ForestWalk> walk_table(bt_forest *f)
         order[i] = i;
         if (f->trees[i]->d_walk) tab[i].w = f->trees[i]->walk;
         tab[i].top_off = kNoTop;
-        // in units of one probe of the top: a sector from the L2 costs about
-        // six, the entry two, the top and the rest of a chunk's work about 16
-        tab[i].cost = 28u + static_cast<uint32_t>(6 * tab[i].w.levels);
+        // Lists of one tree each (51,156 chunks over 10^3, 10^5, 10^6 and 2 * 10^7
+        // keys, 0 to 3 levels) take 19, 28, 34 and 54 us above the launch, a
+        // single chunk's latency grows less than that; in between, so that
+        // both the blocks and the warps in them end together (10,000 batches:
+        // 43.8 us so, 47.2 with the list times as costs, 46.7 with 28 + 6 per
+        // level).
+        const uint64_t entry_bytes = tab[i].w.n / walk_group(f->key_bytes, f->val_bytes) * 64;
+        tab[i].cost = 20u + 8u * static_cast<uint32_t>(tab[i].w.levels) + (entry_bytes > (64u << 20) ? 6u : 0u);
     }
     std::sort(order.begin(), order.end(),
               [&](uint32_t a, uint32_t b) { return tab[a].w.top_bytes < tab[b].w.top_bytes; });

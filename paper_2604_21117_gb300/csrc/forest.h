@@ -51,13 +51,15 @@ cudaError_t forest_run(const bt_forest *f, const bt_batch_desc *batches, uint32_
                        uint32_t host_chunks, uint32_t *plan_ws, const void *q, uint64_t nq, void *out_v,
                        uint8_t *out_f, uint32_t warps, cudaStream_t s, ForestDone done);
 
-// The walk kernel over a work list (arguments as forest_run): every tree of
-// the forest has a walk index or is empty, none has a model.  top_total:
+// The walk kernel over a work list (arguments as forest_run): at most
+// kForestWalkTrees trees, every one has a walk index or is empty, none has a model.  top_total:
 // bytes of the tops that have a place in shared memory.
 cudaError_t forest_walk_run(const ForestWalk *d_tab, uint32_t ntrees, uint32_t top_total, int key_bytes, int val_bytes,
                             const bt_batch_desc *batches, uint32_t nb, const uint32_t *chunk_start, uint32_t host_chunks,
                             const void *q, uint64_t nq, void *out_v, uint8_t *out_f, cudaStream_t s, ForestDone done);
-// The longest device work list the walk kernel plans by itself.
+// The most trees whose table the walk kernel keeps in shared memory, and the
+// longest device work list it plans by itself.
+constexpr uint32_t kForestWalkTrees = 128;
 constexpr uint32_t kForestWalkList = 65536;
 
 // Work-list entries rejected by a kernel: a tree outside the forest, or

@@ -25,7 +25,6 @@ namespace btgb {
 __device__ unsigned long long g_bt_bad_walk_batches;
 
 constexpr uint32_t kWalkForestThreads = 1024;
-constexpr uint32_t kWalkForestTab = 32;  // up to this many trees the table is copied to shared memory
 
 // A position in the list is a cost: entry after entry, each as many chunks as
 // it has times the cost of one.
@@ -59,14 +58,7 @@ __device__ __forceinline__ uint64_t warp_incl_scan(uint64_t x, uint32_t lane)
     return x;
 }
 
-// One row of the work list, an entry per lane, at its positions [first, end).
-struct ListRow {
-    Entry e;
-    uint64_t first, end;
-};
-
-// Shared memory: the tops that have a place (top_total bytes), the first
-// kWalkForestTab table entries, then (lists without chunk offsets) the
+// Shared memory: the tops that have a place (top_total bytes), the table, then (lists without chunk offsets) the
 // positions of the list's rows.
 template <typename K, typename V>
 __global__ void __launch_bounds__(kWalkForestThreads)
@@ -79,9 +71,8 @@ __global__ void __launch_bounds__(kWalkForestThreads)
     __shared__ __align__(8) uint64_t bar;
     __shared__ uint64_t s_scan[32];
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const bool small = ntrees <= kWalkForestTab;
-    ForestWalk *stab = reinterpret_cast<ForestWalk *>(smem + top_total);
-    uint64_t *rows = reinterpret_cast<uint64_t *>(stab + (small ? ntrees : 0u));
+    ForestWalk *tab = reinterpret_cast<ForestWalk *>(smem + top_total);
+    uint64_t *rows = reinterpret_cast<uint64_t *>(tab + ntrees);
     const uint32_t nrows = (nb + 31) / 32;
     if (threadIdx.x == 0) {
         mbar_init(&bar);
@@ -90,10 +81,8 @@ __global__ void __launch_bounds__(kWalkForestThreads)
             if (gtab[i].top_off != kNoTop && gtab[i].w.top_bytes)
                 bulk_g2s(smem + gtab[i].top_off, gtab[i].w.top, gtab[i].w.top_bytes, &bar);
     }
-    if (small)
-        for (uint32_t i = threadIdx.x; i < ntrees * sizeof(ForestWalk) / 8; i += blockDim.x)
-            reinterpret_cast<uint64_t *>(stab)[i] = reinterpret_cast<const uint64_t *>(gtab)[i];
-    const ForestWalk *tab = small ? stab : gtab;
+    for (uint32_t i = threadIdx.x; i < ntrees * sizeof(ForestWalk) / 8; i += blockDim.x)
+        reinterpret_cast<uint64_t *>(tab)[i] = reinterpret_cast<const uint64_t *>(gtab)[i];
     __syncthreads();
     // the work list, the queries and the outputs belong to the previous
     // kernel of the stream until it is done
@@ -102,15 +91,18 @@ __global__ void __launch_bounds__(kWalkForestThreads)
     if (!unit) {
         // row totals (several rows' entries in flight per warp), then their
         // exclusive scan in place (rows[nrows] = the whole list)
-        constexpr int U = 4;
+        constexpr int U = 10;
         for (uint32_t r0 = warp; r0 < nrows; r0 += nw * U) {
             Entry e[U];
 #pragma unroll
             for (int u = 0; u < U; ++u) e[u] = list_entry(batches, (r0 + u * nw) * 32 + lane, nb, tab, ntrees, nq, false);
 #pragma unroll
             for (int u = 0; u < U; ++u) {
-                const uint64_t x = warp_incl_scan(static_cast<uint64_t>(e[u].chunks) * e[u].cost, lane);
-                if (lane == 31 && r0 + u * nw < nrows) rows[r0 + u * nw] = x;
+                // at most 2^27 chunks of a cost below 2^12: two sums below 2^32
+                const uint64_t x = static_cast<uint64_t>(e[u].chunks) * e[u].cost;
+                const uint32_t lo = __reduce_add_sync(0xffffffffu, static_cast<uint32_t>(x) & 0xFFFFFu);
+                const uint32_t hi = __reduce_add_sync(0xffffffffu, static_cast<uint32_t>(x >> 20));
+                if (lane == 0 && r0 + u * nw < nrows) rows[r0 + u * nw] = lo + (static_cast<uint64_t>(hi) << 20);
             }
         }
         __syncthreads();
@@ -152,15 +144,46 @@ __global__ void __launch_bounds__(kWalkForestThreads)
             else
                 hi = mid - 1;
         }
+        // The row, an entry per lane, and in `todo` the entries of it that are
+        // left; the entry at hand, the same in every lane.
         uint32_t row = lo;
-        ListRow R;
+        Entry mine;
+        uint64_t first;  // position of this lane's entry
         auto load_row = [&](uint64_t start) {
-            R.e = list_entry(batches, row * 32 + lane, nb, tab, ntrees, nq, unit);
-            const uint64_t x = static_cast<uint64_t>(R.e.chunks) * R.e.cost;
-            R.end = start + warp_incl_scan(x, lane);
-            R.first = R.end - x;
+            mine = list_entry(batches, row * 32 + lane, nb, tab, ntrees, nq, unit);
+            const uint64_t x = static_cast<uint64_t>(mine.chunks) * mine.cost;
+            const uint64_t end = start + warp_incl_scan(x, lane);
+            first = end - x;
+            return end;
         };
-        load_row(row_pos(row));
+        uint64_t end = load_row(row_pos(row));
+        unsigned todo = __ballot_sync(0xffffffffu, mine.chunks && end > p);
+        Entry e{{0, 0, 0}, 0, 1};
+        uint32_t k = 0;  // the entry's next chunk
+        uint64_t at = 0; // its position
+        bool good = false;
+        auto advance = [&]() -> bool {
+            while (todo == 0) {
+                if (++row >= nrows) return false;
+                end = load_row(__shfl_sync(0xffffffffu, static_cast<unsigned long long>(end), 31));
+                todo = __ballot_sync(0xffffffffu, mine.chunks != 0);
+            }
+            const int src = __ffs(todo) - 1;
+            todo &= todo - 1;
+            e.bd.tree = __shfl_sync(0xffffffffu, mine.bd.tree, src);
+            e.bd.count = __shfl_sync(0xffffffffu, mine.bd.count, src);
+            e.bd.offset = __shfl_sync(0xffffffffu, static_cast<unsigned long long>(mine.bd.offset), src);
+            e.chunks = __shfl_sync(0xffffffffu, mine.chunks, src);
+            e.cost = __shfl_sync(0xffffffffu, mine.cost, src);
+            at = __shfl_sync(0xffffffffu, static_cast<unsigned long long>(first), src);
+            k = 0;
+            good = forest_desc_ok(e.bd, ntrees, nq);
+            if (at < p) {  // the run starts inside this entry
+                k = static_cast<uint32_t>((p - at + e.cost - 1) / e.cost);
+                at += static_cast<uint64_t>(k) * e.cost;
+            }
+            return true;
+        };
         // A chunk's queries, loaded while the chunk before it walks; lanes
         // past the batch's end follow its first query and write nothing.
         struct Chunk {
@@ -169,42 +192,22 @@ __global__ void __launch_bounds__(kWalkForestThreads)
             uint64_t pos;
             K key;
         };
-        uint64_t at = p;  // chunks that start before it are done
         // the next chunk of the run, or false past its end
         auto fetch = [&](Chunk &n) -> bool {
-            unsigned m;
-            for (;;) {  // the entry that holds position `at`, else the first after it
-                m = __ballot_sync(0xffffffffu, R.end > at && R.e.chunks);
-                if (m || row + 1 >= nrows) break;
-                ++row;
-                load_row(__shfl_sync(0xffffffffu, static_cast<unsigned long long>(R.end), 31));
-            }
-            if (!m) return false;
-            const int src = __ffs(m) - 1;
-            const uint64_t first = __shfl_sync(0xffffffffu, static_cast<unsigned long long>(R.first), src);
-            const uint64_t end = __shfl_sync(0xffffffffu, static_cast<unsigned long long>(R.end), src);
-            const uint32_t cost = __shfl_sync(0xffffffffu, R.e.cost, src);
-            // the first chunk of the entry that starts at or after `at`
-            const uint64_t k = at > first ? (at - first + cost - 1) / cost : 0;
-            at = first + k * cost;
-            if (at >= end) {  // `at` lies in the entry's last chunk, which is another warp's
-                at = end;
-                n.live = false;
-                return at < p1;
-            }
+            while (k >= e.chunks)
+                if (!advance()) return false;
             if (at >= p1) return false;
-            at += cost;
-            n.tree = __shfl_sync(0xffffffffu, R.e.bd.tree, src);
-            const uint32_t count = __shfl_sync(0xffffffffu, R.e.bd.count, src);
-            const uint64_t offset = __shfl_sync(0xffffffffu, static_cast<unsigned long long>(R.e.bd.offset), src);
-            n.live = forest_desc_ok(bt_batch_desc{n.tree, count, offset}, ntrees, nq);
-            if (!n.live) {
+            n.live = good;
+            n.tree = e.bd.tree;
+            const uint32_t j0 = k * 32u, j = j0 + lane;
+            ++k;
+            at += e.cost;
+            if (!good) {
                 if (lane == 0) atomicAdd(&g_bt_bad_walk_batches, 1ull);
                 return true;
             }
-            const uint32_t j0 = static_cast<uint32_t>(k) * 32u, j = j0 + lane;
-            n.valid = j < count;
-            n.pos = offset + (n.valid ? j : j0);
+            n.valid = j < e.bd.count;
+            n.pos = e.bd.offset + (n.valid ? j : j0);
             n.key = q[n.pos];
             return true;
         };
@@ -218,9 +221,15 @@ __global__ void __launch_bounds__(kWalkForestThreads)
             V val = static_cast<V>(~static_cast<V>(0));
             bool hit = false;
             if (F.w.n) {
-                const unsigned char *top = F.top_off != kNoTop ? smem + F.top_off : F.w.top;
-                const uint32_t seg = walk_segment<K>(F.w, top, now.key);
-                hit = walk_lookup<K, V>(F.w, walk_entry<K>(F.w, top, seg, now.key), now.key, val);
+                // (two calls, so that each reads the top by its own address space)
+                uint32_t entry;
+                if (F.top_off != kNoTop) {
+                    const unsigned char *top = smem + F.top_off;
+                    entry = walk_entry<K>(F.w, top, walk_segment<K>(F.w, top, now.key), now.key);
+                } else {
+                    entry = walk_entry<K>(F.w, F.w.top, walk_segment<K>(F.w, F.w.top, now.key), now.key);
+                }
+                hit = walk_lookup<K, V>(F.w, entry, now.key, val);
             }
             if (now.valid) {
                 out_v[now.pos] = val;
@@ -255,8 +264,7 @@ static cudaError_t walk_forest_launch(const ForestWalk *tab, uint32_t ntrees, ui
     cudaError_t e = dev_sm_count(&sms);
     if (e == cudaSuccess) e = ensure_dyn_smem(reinterpret_cast<const void *>(kern), 220 * 1024);
     if (e != cudaSuccess) return e;
-    const uint32_t ntab = ntrees <= kWalkForestTab ? ntrees : 0u;
-    const uint32_t smem = top_total + ntab * static_cast<uint32_t>(sizeof(ForestWalk)) +
+    const uint32_t smem = top_total + ntrees * static_cast<uint32_t>(sizeof(ForestWalk)) +
                           (cs ? 0u : ((nb + 31u) / 32u + 1u) * 8u);
     // as many warps per SM as the list has chunks for (a device list: at most
     // as many as batches that do not overlap can have), up to 32
