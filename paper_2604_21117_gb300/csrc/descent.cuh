@@ -344,7 +344,7 @@ __device__ __forceinline__ void model_window(const ModelDev &md, const ModelView
         hat = leaf_from_pred(pl_predict(v.b, v.inv_w, v.slope, v.icpt, md.segments, q), L);
     else
         hat = leaf_from_pred(__fmul_rn(mlp_forward(v.mlp, mlp_x_rank(v.b, v.inv_w, q)), static_cast<float>(L - 1)), L);
-    const uint32_t er = __ldg(md.errs + err_range(hat, L));
+    const uint32_t er = __ldg(md.errs + div_by(static_cast<uint64_t>(hat) * kErrRanges, L, md.leaves_inv));
     lo = hat > er ? hat - er : 0u;
     hi = (static_cast<uint64_t>(hat) + er < L) ? hat + er : L - 1;
 }

@@ -415,6 +415,7 @@ extern "C" bt_status bt_model_train(const bt_tree *tree, const bt_learn_opts *op
     md.kind = opts->kind;
     md.segments = S;
     md.leaves = static_cast<uint32_t>(L);
+    md.leaves_inv = ~0ull / L;
     md.leaf_max = base + off_lmax;
     md.errs = reinterpret_cast<const uint32_t *>(base + 256);
     md.kmin = t.kmin;

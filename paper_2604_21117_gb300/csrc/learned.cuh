@@ -48,6 +48,20 @@ __host__ __device__ __forceinline__ uint32_t err_range(uint32_t hat, uint32_t L)
     return static_cast<uint32_t>((static_cast<uint64_t>(hat) * kErrRanges) / L);
 }
 
+// x / d by m = floor((2^32 - 1) / d), and the same for a numerator below 2^40
+// by m = floor((2^64 - 1) / d): the product is at most one short.
+__device__ __forceinline__ uint32_t div_by(uint32_t x, uint32_t d, uint32_t m)
+{
+    const uint32_t q = __umulhi(x, m);
+    return x - q * d >= d ? q + 1 : q;
+}
+
+__device__ __forceinline__ uint32_t div_by(uint64_t x, uint32_t d, uint64_t m)
+{
+    const uint64_t q = __umul64hi(x, m);
+    return static_cast<uint32_t>(x - q * d >= d ? q + 1 : q);
+}
+
 // Everything the search kernel needs to use a model, passed by value.
 struct ModelDev {
     int kind;
@@ -55,6 +69,7 @@ struct ModelDev {
     uint32_t err;           // max |leaf_hat - leaf| over the stored keys
     const uint32_t *errs;   // the same maximum per range of leaf_hat (kErrRanges ranges)
     uint32_t leaves;        // L
+    uint64_t leaves_inv;    // floor((2^64 - 1) / L)
     const uint64_t *b;      // PL breakpoints (as uint64 whatever the key width)
     const float *inv_w;     // PL
     const float *slope;     // PL
@@ -124,15 +139,17 @@ __device__ __forceinline__ float mlp_x(uint64_t q, uint64_t kmin, uint64_t kmax,
 
 // Network output for input x (parameters p, any address space, 16-byte
 // aligned).  A lane evaluates the whole network: the second layer's rows are
-// read four weights at a time, so that a warp's loads (one broadcast each)
-// stay below its multiplications.
+// read four weights at a time.  Two rows at a time: at 1024 lookups a warp
+// has an SM to itself and the loop's code is fetched for it alone (searches
+// of 2^24 keys, 1 / 2 / 4 / 8 rows: 8.1 / 7.9 / 9.0 / 8.6 us; at 2^20 lookups
+// 125 / 125 / 132 / 129, bound by the broadcast weights' way to registers).
 __device__ __forceinline__ float mlp_forward(const float *p, float x)
 {
     float h1[kMlpH];
 #pragma unroll
     for (int j = 0; j < kMlpH; ++j) h1[j] = fmaxf(fmaf(p[kOffW1 + j], x, p[kOffB1 + j]), 0.0f);
     float y = p[kOffB3];
-#pragma unroll 8
+#pragma unroll 2
     for (int j = 0; j < kMlpH; ++j) {
         const float4 *w = reinterpret_cast<const float4 *>(p + kOffW2 + j * kMlpH);
         float z = p[kOffB2 + j];

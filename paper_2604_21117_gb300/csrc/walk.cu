@@ -357,6 +357,7 @@ constexpr int walk_threads()
 struct WalkModel {
     ModelDev md;
     uint64_t leaf_base, leaf_rem;  // keys per leaf, leaves with one more
+    uint32_t span_inv;             // floor((2^32 - 1) / entries per segment)
 };
 
 // The model's parameters in shared memory behind the top, each array rounded
@@ -369,19 +370,19 @@ __host__ __device__ inline uint32_t walk_model_bytes(const ModelDev &m)
     return 0u;
 }
 
-// Where the parameters are, and (one thread, `copy`) their bulk copies.
+// Where the parameters lie behind the top, and (one thread, `bar` given) the
+// bulk copies that bring them there.
 template <int MODEL>
-__device__ __forceinline__ ModelView walk_model(const ModelDev &md, unsigned char *msm, uint64_t *bar, bool copy)
+__device__ __forceinline__ ModelView walk_model(const ModelDev &md, unsigned char *msm, uint64_t *bar = nullptr)
 {
-    ModelView v{md.b, md.inv_w, md.slope, md.icpt, md.mlp};
-    if (walk_model_bytes(md) == 0) return v;
     auto put = [&](const void *src, uint32_t bytes) {
         const uint32_t padded = (bytes + 15u) / 16u * 16u;
         unsigned char *dst = msm;
-        if (copy) bulk_g2s(dst, src, padded, bar);
+        if (bar) bulk_g2s(dst, src, padded, bar);
         msm += padded;
         return dst;
     };
+    ModelView v{};
     const uint32_t S = MODEL == kModelPL ? md.segments : kMlpStage1;
     v.b = reinterpret_cast<const uint64_t *>(put(md.b, S * 8u));
     v.inv_w = reinterpret_cast<const float *>(put(md.inv_w, S * 4u));
@@ -433,9 +434,9 @@ __global__ void __launch_bounds__(walk_threads<MODEL>())
         mbar_init(&bar);
         mbar_arrive_expect_tx(&bar, w.top_bytes + (MODEL == kModelNone ? 0u : walk_model_bytes(m.md)));
         if (w.top_bytes) bulk_g2s(smem, w.top, w.top_bytes, &bar);
+        if constexpr (MODEL != kModelNone)
+            if (walk_model_bytes(m.md)) walk_model<MODEL>(m.md, smem + w.top_bytes, &bar);
     }
-    ModelView mv{};
-    if constexpr (MODEL != kModelNone) mv = walk_model<MODEL>(m.md, smem + w.top_bytes, &bar, threadIdx.x == 0);
     pdl_wait();
     const uint32_t chunks = (nq + 31) / 32;
     const uint32_t c1 = static_cast<uint32_t>(static_cast<uint64_t>(chunks) * (blockIdx.x + 1) / gridDim.x);
@@ -475,11 +476,16 @@ __global__ void __launch_bounds__(walk_threads<MODEL>())
             constexpr uint32_t G = walk_group(sizeof(K), sizeof(V));
             const W *sep = reinterpret_cast<const W *>(smem);
             uint32_t lo, hi;
-            model_window<MODEL>(m.md, mv, static_cast<uint64_t>(key), lo, hi);
+            // (two calls, so that each reads the parameters by their own address space)
+            if (MODEL == kModelMLP || walk_model_bytes(m.md))
+                model_window<MODEL>(m.md, walk_model<MODEL>(m.md, smem + w.top_bytes), static_cast<uint64_t>(key), lo, hi);
+            else
+                model_window<MODEL>(m.md, ModelView{m.md.b, m.md.inv_w, m.md.slope, m.md.icpt, m.md.mlp},
+                                    static_cast<uint64_t>(key), lo, hi);
             // first key of leaf lo, last key of leaf hi, as entries, as segments
             const uint64_t r0 = lo * m.leaf_base + (lo < m.leaf_rem ? lo : m.leaf_rem);
             const uint64_t r1 = (hi + 1ull) * m.leaf_base + (hi + 1ull < m.leaf_rem ? hi + 1ull : m.leaf_rem) - 1;
-            const uint32_t s0 = static_cast<uint32_t>(r0 / G) / w.span, s1 = static_cast<uint32_t>(r1 / G) / w.span;
+            const uint32_t s0 = div_by(static_cast<uint32_t>(r0 / G), w.span, m.span_inv), s1 = div_by(static_cast<uint32_t>(r1 / G), w.span, m.span_inv);
             // proven by the separators on both sides, else the whole top searched
             if ((s0 == 0 || sep[s0 - 1] < word) && (s1 + 1 >= w.segs || !(sep[s1] < word)))
                 seg = walk_segment_in<W>(sep, s0, s1, word);
@@ -519,6 +525,7 @@ static cudaError_t walk_launch(const bt_tree *t, const ModelDev *md, const void 
         m.md = *md;
         m.leaf_base = t->dev.cbase[leaf];
         m.leaf_rem = t->dev.crem[leaf];
+        m.span_inv = ~0u / w.span;
     }
     // one block per SM with as many warps as its share of the chunks
     constexpr uint64_t kWarps = walk_threads<MODEL>() / 32;
