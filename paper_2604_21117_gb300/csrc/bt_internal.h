@@ -104,10 +104,11 @@ void set_pin_levels(DevTree &d, const bt_info &info, uint32_t budget);
 // Host-side launch facts, cached per device and safe to call from any
 // thread: the current device's SM count, resident blocks per SM of a kernel
 // at a block shape, and the kernel's dynamic shared-memory limit raised to
-// `bytes` (once per device and kernel).
+// `bytes` (once per device and kernel), with its preferred share of shared
+// memory (percent) when `carveout` is not negative.
 cudaError_t dev_sm_count(int *sms);
 cudaError_t blocks_per_sm(const void *kern, int threads, int dyn_smem, int *out);
-cudaError_t ensure_dyn_smem(const void *kern, int bytes);
+cudaError_t ensure_dyn_smem(const void *kern, int bytes, int carveout = -1);
 
 // Poll limit of the first bounded wait in the descent (bt_debug_set_wait_polls).
 uint32_t first_wait_polls();

@@ -140,7 +140,7 @@ cudaError_t blocks_per_sm(const void *kern, int threads, int dyn_smem, int *out)
     return cudaSuccess;
 }
 
-cudaError_t ensure_dyn_smem(const void *kern, int bytes)
+cudaError_t ensure_dyn_smem(const void *kern, int bytes, int carveout)
 {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -150,6 +150,8 @@ cudaError_t ensure_dyn_smem(const void *kern, int bytes)
     auto it = g_dyn.find(key);
     if (it != g_dyn.end() && it->second >= bytes) return cudaSuccess;
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess && carveout >= 0)
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, carveout);
     if (e != cudaSuccess) return e;
     g_dyn[key] = bytes;
     return cudaSuccess;

@@ -68,7 +68,7 @@ constexpr int kForestSmemMax = 200 * 1024;
 // 10^3, 10^5, 10^6 and 2 * 10^7 uint64 keys, with tops searched by bisection
 // (146 KB): 58.9 us with all of them there, 71.7 with 96 KB (the largest
 // tree's top through L1), 68.9 with none.
-constexpr uint32_t kWalkTopBudget = 160 * 1024;
+constexpr uint32_t kWalkTopBudget = 128 * 1024;
 
 __host__ __device__ inline uint32_t forest_desc_chunks(const bt_batch_desc &bd, uint32_t ntrees, uint64_t nq,
                                                        int lq)
@@ -566,7 +566,7 @@ static std::vector<ForestWalk> walk_table(bt_forest *f)
         // both the blocks and the warps in them end together (10,000 batches:
         // 43.8 us so, 47.2 with the list times as costs, 46.7 with 28 + 6 per
         // level).
-        const uint64_t entry_bytes = tab[i].w.n / walk_group(f->key_bytes, f->val_bytes) * 64;
+        const uint64_t entry_bytes = tab[i].w.n / walk_group(f->key_bytes, f->val_bytes) * 32;
         tab[i].cost = 20u + 8u * static_cast<uint32_t>(tab[i].w.levels) + (entry_bytes > (64u << 20) ? 6u : 0u);
     }
     std::sort(order.begin(), order.end(),

@@ -262,7 +262,7 @@ static cudaError_t walk_forest_launch(const ForestWalk *tab, uint32_t ntrees, ui
     auto kern = k_forest_walk<K, V>;
     int sms = 0;
     cudaError_t e = dev_sm_count(&sms);
-    if (e == cudaSuccess) e = ensure_dyn_smem(reinterpret_cast<const void *>(kern), 220 * 1024);
+    if (e == cudaSuccess) e = ensure_dyn_smem(reinterpret_cast<const void *>(kern), 220 * 1024, kWalkCarveout);
     if (e != cudaSuccess) return e;
     const uint32_t smem = top_total + ntrees * static_cast<uint32_t>(sizeof(ForestWalk)) +
                           (cs ? 0u : ((nb + 31u) / 32u + 1u) * 8u);

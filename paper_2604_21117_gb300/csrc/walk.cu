@@ -43,9 +43,10 @@ __global__ void k_walk_entries(LeafView lv, uint64_t n, uint64_t slots, unsigned
     constexpr uint32_t G = walk_group(sizeof(K), sizeof(V));
     for (uint64_t i = blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x; i < slots;
          i += static_cast<uint64_t>(gridDim.x) * blockDim.x) {
-        unsigned char *p = entries + i / G * 64u;
+        constexpr uint32_t B = walk_entry_bytes(sizeof(K));
+        unsigned char *p = entries + i / G * B;
         K *k = reinterpret_cast<K *>(p) + i % G;
-        V *v = reinterpret_cast<V *>(p + 32) + i % G;
+        V *v = reinterpret_cast<V *>(p + B / 2) + i % G;
         if (i < n) {
             const uint64_t s = leaf_slot(lv, i);
             *k = static_cast<const K *>(lv.keys)[s];
@@ -256,8 +257,8 @@ cudaError_t walk_build(bt_tree *t, const void *h_keys, cudaStream_t s)
     const LeafView lv{d.keys[leaf], d.vals, d.cbase[leaf], d.crem[leaf], static_cast<uint32_t>(d.m)};
     cudaError_t e = cudaSuccess;
     // coded levels: one where it leaves at most kWalkSegs segments, else two;
-    // none where codes tie; then levels of full words down to kWalkMaxSegs
-    // (without codes kWalkMaxSegs / 2, as those trees' tops measured best)
+    // none where codes tie; then levels of full words down to walk_max_segs
+    // (without codes half of it)
     uint64_t segs = E, span = 1, count[kWalkLevels];
     if (E > kWalkSegs) {
         w.coded = (E + kCodeFan - 1) / kCodeFan <= kWalkSegs ? 1 : 2;
@@ -277,7 +278,7 @@ cudaError_t walk_build(bt_tree *t, const void *h_keys, cudaStream_t s)
         span *= kCodeFan;
     }
     w.levels = w.coded;
-    while (segs > (w.coded ? kWalkMaxSegs : kWalkMaxSegs / 2)) {
+    while (segs > (w.coded ? walk_max_segs(kb) : walk_max_segs(kb) / 2)) {
         segs = (segs + F - 1) / F;
         span *= F;
         ++w.levels;
@@ -305,7 +306,7 @@ cudaError_t walk_build(bt_tree *t, const void *h_keys, cudaStream_t s)
     }
     bytes = (bytes + 255) & ~255ull;
     const uint64_t ent_off = bytes;
-    bytes += E * 64;
+    bytes += E * walk_entry_bytes(kb);
     size_t free_b = 0, total_b = 0;
     e = cudaMemGetInfo(&free_b, &total_b);
     if (e != cudaSuccess) return e;
@@ -403,14 +404,15 @@ __device__ __forceinline__ ModelView walk_model(const ModelDev &md, unsigned cha
 //
 // What bounds it: divergent reads.  A warp's read of one sector per lane
 // occupies an SM for 34 cycles when it comes from the L2 and 20 when it hits
-// L1, whatever part of the sector is used; a probe of the top in shared
-// memory for 6; and 2^20 reads of random entries of 64 bytes take 18 us from
-// memory by themselves.  Over 2^24 uint64 keys a query is about six probes,
-// two coded nodes, an entry's keys and one value: 33.6 us for 2^20 queries
-// with three trees in turn (31.5 for one).  Before the walk, the partition
-// and the level-wise descent: 92.4 us; with four nodes of full words under a
-// top searched by bisection (13 probes): 41.6; with the top's tables 41.2.
-// For 32-byte keys (2^20 keys) 113, 38.6, 36.9, now 31.4 us.
+// L1, whatever part of the sector is used (about 4.7 us per 2^20 queries); a
+// probe of the top in shared memory for 6; and 2^20 reads of random entries
+// take 18 us from memory by themselves.  Over 2^24 uint64 keys a query is
+// about six probes, three nodes and an entry: 32.7 us for 2^20 queries with
+// three trees in turn (30.2 for one).  Before the walk, the partition and
+// the level-wise descent: 92.4 us; with four nodes of full words under a top
+// searched by bisection (13 probes) and entries of 64 bytes: 41.6; with the
+// top's tables 41.2; with coded nodes 33.4.  For 32-byte keys (2^20 keys) 113,
+// 38.6, 36.9, now 32.3 us; over 10^6 uint64 keys 61, 25.1, -, now 17.5.
 // 1024 threads on one SM: two blocks (of 1024, 768 or 512) hold two copies
 // of the top and gain nothing from the additional warps (2^20 queries over
 // 2^24 keys, full-word nodes: 42.3, 43.5 and 51.4 us against 40.4).
@@ -516,7 +518,7 @@ static cudaError_t walk_launch(const bt_tree *t, const ModelDev *md, const void 
     constexpr int kMaxModel = MODEL == kModelNone ? 0 : static_cast<int>(kModelSmemSegments) * 20 + 64;
     int sms = 0;
     cudaError_t e = dev_sm_count(&sms);
-    if (e == cudaSuccess) e = ensure_dyn_smem(reinterpret_cast<const void *>(kern), kMaxTop + kMaxModel);
+    if (e == cudaSuccess) e = ensure_dyn_smem(reinterpret_cast<const void *>(kern), kMaxTop + kMaxModel, kWalkCarveout);
     if (e != cudaSuccess) return e;
     WalkModel m;
     memset(&m, 0, sizeof(m));

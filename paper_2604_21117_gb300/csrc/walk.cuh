@@ -7,7 +7,8 @@
 // SMs.  The walk index holds the same keys and values a second time in the
 // form that costs the fewest sectors per query:
 //
-//   top      the largest keys of up to 2^14 segments of equal length,
+//   top      the largest keys of up to 15360 segments of equal length (25600
+//            for 32-bit keys),
 //            ascending, and two tables that narrow the search
 //            among them to a few: the octave of x = key - smallest key (its
 //            leading one) gives a range of bins, as many as the octave has
@@ -32,13 +33,12 @@
 //            Node i has the children FAN i .. FAN i + SEP of the next level
 //            (17 i .. 17 i + 16), separator j stands for the largest key under
 //            child j, all-ones where child j + 1 does not exist;
-//   entries  64 bytes each, the children of the last level.  Integer keys: G
-//            consecutive keys (bytes 0..31, unused slots all-ones) and their
-//            values (bytes 32..63), G = 32 / max(key, value bytes); the keys
-//            are packed densely, entry e holding ranks G e .. G e + G - 1.
-//            Memory is read 64 bytes at a time, so a query costs one such
-//            access for its key and its value together.
-//            32-byte keys: one key (four words, as Key32) and its value.
+//   entries  the children of the last level.  Integer keys: one sector, G =
+//            32 / (key + value bytes) consecutive keys (bytes 0..15, unused
+//            slots all-ones) and their values (bytes 16..31), so that one read
+//            brings a query's key and its value; the keys are packed densely,
+//            entry e holding ranks G e .. G e + G - 1.  32-byte keys: 64
+//            bytes, one key (four words, as Key32) and its value.
 //
 // 32-byte keys are walked by one 64-bit word, the 8 bytes after the bytes all
 // keys share: a query between the smallest and the largest key shares those
@@ -69,20 +69,33 @@ constexpr uint32_t walk_fan(int key_bytes) { return key_bytes == 4 ? 9u : 5u; }
 constexpr uint32_t kCodeFan = 17;
 // Segments at most: above 2^12 a second coded level is cheaper than the
 // larger top (its copy, and the room it takes from L1), and a level of full
-// words dearer than a top of up to 2^14.
-constexpr uint32_t kWalkSegs = 4096, kWalkMaxSegs = 16384;
+// words dearer than a top of up to 160 KB (2^20 queries of 2^23 uint64 keys,
+// 148 KB of top: 23.5 us, with a level instead and a 29 KB top 25.4).
+constexpr uint32_t kWalkSegs = 4096;
+constexpr uint32_t walk_max_segs(int key_bytes) { return key_bytes == 4 ? 25600 : 15360; }
 // Bytes of the largest top: separators, at most one bin each and one per
 // octave besides, the octaves, padding.
 constexpr int walk_max_top(int key_bytes)
 {
-    return static_cast<int>(kWalkMaxSegs) * ((key_bytes == 4 ? 4 : 8) + 2) + 64 * 2 + 64 * 8 + 64;
+    return static_cast<int>(walk_max_segs(key_bytes)) * ((key_bytes == 4 ? 4 : 8) + 2) + 64 * 2 + 64 * 8 + 64;
 }
 
-// Keys per entry.
+// Keys and bytes per entry.
 __host__ __device__ constexpr uint32_t walk_group(int key_bytes, int val_bytes)
 {
-    return key_bytes > 8 ? 1u : 32u / static_cast<uint32_t>(key_bytes > val_bytes ? key_bytes : val_bytes);
+    return key_bytes > 8 ? 1u : 32u / static_cast<uint32_t>(key_bytes + val_bytes);
 }
+__host__ __device__ constexpr uint32_t walk_entry_bytes(int key_bytes) { return key_bytes > 8 ? 64u : 32u; }
+
+// The walk kernels ask for no more shared memory on an SM than their one
+// block needs: misses in flight are held in L1 lines, so L1 is what bounds
+// them.  Left to the runtime, which makes room for as many blocks as the SM
+// could hold, a top of 100 to 114 KB (two blocks fit) left 28 KB of L1, and
+// 2^20 uniform queries of 2 * 10^7 uint32 keys took 51 us instead of 22; with
+// 228 / 196 / 164 / 132 / 100 KB of shared memory for the 58 KB top of 2^24
+// uint64 keys 2^20 queries take 72 / - / 42.0 / 35.5 / 33.3 us, with as much
+// as needed 32.7.
+constexpr int kWalkCarveout = 0;  // cudaSharedmemCarveoutMaxL1
 
 // One 32-byte sector as words.
 template <typename W>
@@ -234,35 +247,50 @@ __device__ __forceinline__ uint32_t walk_entry(const WalkDev &w, const unsigned 
     return node;
 }
 
-// An entry's keys as loaded, whether its largest lies below q, and q's place
-// among them (G: not there).
-template <typename K>
-struct EntryKeys {
-    Sector<typename WalkWord<K>::type> s;
-    __device__ __forceinline__ explicit EntryKeys(const unsigned char *p) : s(ld_sector<typename WalkWord<K>::type>(p))
+// An entry as loaded: whether its keys all lie below q, q's place among them
+// (G: not there), and the value there (integer keys).
+template <typename K, typename V>
+struct WalkEntry {
+    static constexpr uint32_t G = walk_group(sizeof(K), sizeof(V));
+    Sector<uint32_t> s;
+    __device__ __forceinline__ WalkEntry(const WalkDev &w, uint64_t e)
+        : s(ld_sector<uint32_t>(w.entries + e * walk_entry_bytes(sizeof(K))))
     {
     }
-    __device__ __forceinline__ Key32 key32() const { return Key32{{s.w[0], s.w[1], s.w[2], s.w[3]}}; }
-    template <uint32_t G>
-    __device__ __forceinline__ bool below(const K &q) const
+    __device__ __forceinline__ uint64_t word(uint32_t i) const
+    {
+        return s.w[2 * i] | static_cast<uint64_t>(s.w[2 * i + 1]) << 32;
+    }
+    __device__ __forceinline__ K key(uint32_t j) const
     {
         if constexpr (sizeof(K) > 8)
-            return key32() < q;
+            return Key32{{word(0), word(1), word(2), word(3)}};
+        else if constexpr (sizeof(K) == 8)
+            return word(j);
         else
-            return s.w[G - 1] < q;
+            return s.w[j];
     }
-    template <uint32_t G>
+    __device__ __forceinline__ bool below(const K &q) const { return key(G - 1) < q; }
     __device__ __forceinline__ uint32_t find(const K &q) const
     {
         uint32_t at = G;
-        if constexpr (sizeof(K) > 8) {
-            if (key32() == q) at = 0;
-        } else {
 #pragma unroll
-            for (uint32_t j = G; j-- > 0;)
-                if (s.w[j] == q) at = j;
-        }
+        for (uint32_t j = G; j-- > 0;)
+            if (key(j) == q) at = j;
         return at;
+    }
+    __device__ __forceinline__ V value(uint32_t at) const
+    {
+        V v = 0;
+#pragma unroll
+        for (uint32_t j = 0; j < G; ++j)
+            if (at == j) {
+                if constexpr (sizeof(V) == 8)
+                    v = word(2 + j);
+                else
+                    v = s.w[4 + j];
+            }
+        return v;
     }
 };
 
@@ -271,42 +299,48 @@ struct EntryKeys {
 template <typename K, typename V>
 __device__ __forceinline__ bool walk_lookup(const WalkDev &w, uint32_t e, const K &q, V &val)
 {
-    constexpr uint32_t G = walk_group(sizeof(K), sizeof(V));
-    const unsigned char *p = w.entries + static_cast<uint64_t>(e) * 64u;
-    const EntryKeys<K> k(p);
+    using Entry = WalkEntry<K, V>;
+    constexpr uint32_t G = Entry::G;
     val = static_cast<V>(~static_cast<V>(0));
-    uint32_t at = k.template find<G>(q);
+    uint64_t at_e = e;
+    const Entry x(w, e);
+    uint32_t at = x.find(q);
     if (at < G) {
-        // the last entry's unused slots hold all-ones, which may be the query
-        if (static_cast<uint64_t>(e) * G + at >= w.n) return false;
-        // read only now that its place is known, although the entry's two
-        // sectors could be asked for together: the keys' read has brought
-        // both to the L2, and a second read that waits for memory costs more
-        // than one that hits (2^20 over 2^24 keys: 34.5 us together, 33.6 so)
-        val = ld_key(reinterpret_cast<const V *>(p + 32) + at);
-        return true;
+        if constexpr (sizeof(K) <= 8) val = x.value(at);
+    } else {
+        if (!x.below(q)) return false;
+        // gallop to the first entry that is not below q
+        const uint64_t E = (w.n + G - 1) / G;
+        uint64_t lo = at_e + 1, step = 1;
+        while (lo + step <= E && Entry(w, lo + step - 1).below(q)) {
+            lo += step;
+            step *= 2;
+        }
+        uint64_t hi = lo + step - 1 < E ? lo + step - 1 : E;
+        while (lo < hi) {
+            const uint64_t mid = (lo + hi) / 2;
+            if (Entry(w, mid).below(q))
+                lo = mid + 1;
+            else
+                hi = mid;
+        }
+        if (lo >= E) return false;
+        const Entry y(w, lo);
+        at = y.find(q);
+        if (at == G) return false;
+        if constexpr (sizeof(K) <= 8) val = y.value(at);
+        at_e = lo;
     }
-    if (!k.template below<G>(q)) return false;
-    // gallop to the first entry that is not below q
-    const uint64_t E = (w.n + G - 1) / G;
-    uint64_t lo = static_cast<uint64_t>(e) + 1, step = 1;
-    while (lo + step <= E && EntryKeys<K>(w.entries + (lo + step - 1) * 64u).template below<G>(q)) {
-        lo += step;
-        step *= 2;
+    // the last entry's unused slots hold all-ones, which may be the query
+    if (at_e * G + at >= w.n) {
+        val = static_cast<V>(~static_cast<V>(0));
+        return false;
     }
-    uint64_t hi = lo + step - 1 < E ? lo + step - 1 : E;
-    while (lo < hi) {
-        const uint64_t mid = (lo + hi) / 2;
-        if (EntryKeys<K>(w.entries + mid * 64u).template below<G>(q))
-            lo = mid + 1;
-        else
-            hi = mid;
-    }
-    if (lo >= E) return false;
-    p = w.entries + lo * 64u;
-    at = EntryKeys<K>(p).template find<G>(q);
-    if (at == G || lo * G + at >= w.n) return false;
-    val = ld_key(reinterpret_cast<const V *>(p + 32) + at);
+    // a 32-byte key's value is read only now: the key's read has brought the
+    // entry's other sector to the L2 too, and a second read that waits for
+    // memory costs more than one that hits (2^20 keys: 32.5 us both at once,
+    // 31.4 so)
+    if constexpr (sizeof(K) > 8) val = ld_key(reinterpret_cast<const V *>(w.entries + at_e * 64u + 32));
     return true;
 }
 
