@@ -1118,9 +1118,10 @@ def run_ours(a):
             and a.pin < 0 and a.sort_bits < 0):
         traffic = NCU_DESCEND_TRAFFIC["bytes_per_launch"]
     step_gbs = statistics.fmean(node_bytes) / (total_s / K) / 1e9  # per batch, at the whole job's rate
-    sort_k = bt.bt_sort_launches(tree.handle, B, sort_bits)
-    # our kernels per step: the partition's kernels, then the descent
-    launches_per_step = sort_k + 1
+    # our kernels per step: one walk of the batch as given, or the partition's
+    # kernels and the descent
+    walk = sort_bits <= 0 and a.staging == 2 and a.lane_queries == 1 and a.ballot == 0
+    launches_per_step = 1 if walk else bt.bt_sort_launches(tree.handle, B, sort_bits) + 1
     sdev = sorted(step_ms)
 
     line = {
