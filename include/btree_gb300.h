@@ -131,13 +131,15 @@ typedef struct bt_info {
  * after the bytes all keys share).
  *
  * Beside the image, in an allocation of its own that bt_info does not count,
- * the device keeps a walk index: the keys and values once more in 64-byte
- * entries under 32-byte nodes, through which batches are searched as given
- * (see bt_search_opts.sort_bits).  It takes about 17 bytes per 64-bit key
- * and value (8.5 for 32-bit ones, 66 per 32-byte key), more where keys crowd
- * (up to 20, 9 and 72), and is left out when
- * that is more than a quarter of the free device memory; searches are then
- * partitioned and descend the tree as bt_sort_bits says.
+ * the device keeps a walk index: the keys and values once more in one-sector
+ * entries (32-byte keys: 64 bytes each) under one-sector nodes, through which
+ * batches are searched as given (see bt_search_opts.sort_bits).  It takes
+ * about 18 bytes per 64-bit key and value (9 for 32-bit ones, 66 per 32-byte
+ * key), more where keys crowd (up to 20, 10 and 72), and is left out when
+ * that is more than a quarter of the free device memory, or where the 8 bytes
+ * after the bytes all 32-byte keys share are the same for hundreds of keys on
+ * end; searches are then partitioned and descend the tree as bt_sort_bits
+ * says.
  *
  * Errors: BT_ERR_ARG, BT_ERR_FANOUT, BT_ERR_UNSORTED, BT_ERR_DUPLICATE,
  * BT_ERR_NOMEM, BT_ERR_CUDA.  *out is set only on BT_OK.
@@ -176,11 +178,10 @@ typedef struct bt_search_opts {
      * tree has none, d_fetch_counts is set, or another descent than the
      * pipelined one with the binary-search rank has been chosen for it
      * (bt_tree_set_staging, bt_tree_set_lane_queries, bt_tree_set_descent);
-     * then -1 partitions on
-     * bt_sort_bits bits (none below 786432 queries -- 393216 for 32-byte
-     * keys -- and none for a tree whose device image is at most a quarter of
-     * the L2: the partition pays for itself only when the batch is large and
-     * leaf blocks do not stay in the L2 between batches). */
+     * then -1 partitions on bt_sort_bits bits (none below 786432 queries --
+     * 393216 for 32-byte keys -- and none for a tree whose device image is at
+     * most a quarter of the L2: the partition pays for itself only when the
+     * batch is large and leaf blocks do not stay in the L2 between batches). */
     int32_t sort_bits;
     /* If non-NULL: device array of `height` counters to which the search
      * adds, per level, how many node key blocks it fetched -- the quantity
@@ -264,15 +265,16 @@ bt_status bt_sort_batch(const bt_tree *tree, const void *d_queries, uint64_t nq,
                         void *d_sorted_queries, uint32_t *d_sorted_index, void *d_workspace,
                         uint64_t ws_bytes, bt_stream stream);
 
-/* Number of kernels the partition of bt_sort_batch / bt_search_batch
+/* Number of kernels the partition of bt_sort_batch, and of a bt_search_batch
+ * that does not go through the walk index (see bt_search_opts.sort_bits),
  * launches for this tree, batch size and sort_bits (0 = no partition; it
  * also issues one cudaMemsetAsync of its bucket counters).  -1 on a NULL
  * tree. */
 int32_t bt_sort_launches(const bt_tree *tree, uint64_t nq, int32_t sort_bits);
 
-/* Bits of the bucket number f that bt_sort_batch / bt_search_batch order a
- * batch of nq queries on, for this sort_bits (-1 = the library's choice);
- * 0 = no partition.  -1 on a NULL tree.  No counterpart in the paper. */
+/* Bits of the bucket number f that bt_sort_batch, and a bt_search_batch that
+ * does not go through the walk index, order a batch of nq queries on, for
+ * this sort_bits (-1 = the library's choice); 0 = no partition.  -1 on a NULL tree.  No counterpart in the paper. */
 int32_t bt_sort_bits(const bt_tree *tree, uint64_t nq, int32_t sort_bits);
 
 /*
@@ -537,6 +539,8 @@ bt_status bt_tree_set_l2_window(bt_tree *tree, uint64_t max_bytes);
  * (Sec. V-B, Fig. 7), here on the device.  Results do not change; a single
  * stream runs slower with the caps.  The partition stays one cooperative
  * launch (all of its blocks resident before any passes a grid barrier).
+ * Batches searched through the walk index run one block per SM whatever the
+ * caps; two of them in flight overlap without any.
  * Not thread-safe with searches running on the tree.  No counterpart in
  * the paper's kernel.  BT_ERR_ARG above 32. */
 bt_status bt_tree_set_corun(bt_tree *tree, uint32_t descent_blocks_per_sm, uint32_t partition_blocks_per_sm);

@@ -377,7 +377,8 @@ cudaError_t descend_paper_layout(const DevTree &t, const PaperTree &p, const voi
 // Builds the walk index of a tree whose image is on the device (h_keys: the
 // sorted keys it was built from), in an allocation of its own.  Leaves the tree without one (and returns
 // cudaSuccess) when the index would take more than a quarter of the free
-// device memory, or the key count exceeds what its node numbers hold.
+// device memory, the key count exceeds what its node numbers hold, or
+// 32-byte keys share the words it walks in long runs.
 cudaError_t walk_build(bt_tree *tree, const void *h_keys, cudaStream_t s);
 // Search of a batch as given through the walk index; md: with a model of the
 // tree (integer keys).

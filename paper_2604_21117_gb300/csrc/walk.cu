@@ -131,6 +131,28 @@ static unsigned fill_grid(uint64_t items)
     return static_cast<unsigned>(g < 65536 ? (g > 0 ? g : 1) : 65536);
 }
 
+// Sum over the keys of the probes that a search for each needs to come from
+// the first key with its word to itself (two per doubling of the distance).
+__global__ void k_walk_runs(LeafView lv, uint64_t n, int p0, unsigned long long *__restrict__ probes)
+{
+    unsigned long long mine = 0;
+    for (uint64_t i = blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x; i < n;
+         i += static_cast<uint64_t>(gridDim.x) * blockDim.x) {
+        const uint64_t word = walk_word<Key32>(lv, i, p0);
+        if (i == 0 || walk_word<Key32>(lv, i - 1, p0) != word) continue;
+        uint64_t lo = 0, hi = i;  // the first key whose word is not below
+        while (lo < hi) {
+            const uint64_t mid = (lo + hi) / 2;
+            if (walk_word<Key32>(lv, mid, p0) < word)
+                lo = mid + 1;
+            else
+                hi = mid;
+        }
+        mine += 2u * static_cast<unsigned>(64 - __clzll(static_cast<long long>(i - lo)));
+    }
+    if (mine) atomicAdd(probes, mine);
+}
+
 template <typename K>
 static cudaError_t build_levels(const WalkDev &w, const LeafView &lv, uint64_t E, uint32_t G, const uint64_t *count,
                                 unsigned char *nodes, cudaStream_t s)
@@ -159,24 +181,31 @@ static cudaError_t build_levels(const WalkDev &w, const LeafView &lv, uint64_t E
 // dense runs of 40 (a tenth, half, one and two percent of the entries tie):
 // 30.1 / 31.7 / 33.3 / 36.0 us through codes, 31.9 through full words at any
 // share (27.9 and 31.9 without runs).
+// *skip: 32-byte keys whose words tie in runs so long that walking on from
+// the first of one costs more than the descent, on average 16 probes (2^20
+// keys in runs of 30 / 200 / 5000, 2^20 lookups: 70 / 97 / 145 us, by the
+// partition and descent 114 / 131 / 130; 1000 lookups: 6.9 / 8.6 / 11.4 us
+// against 9.0 / 9.4 / 9.8).
 template <typename K>
 static cudaError_t codes_tie(const LeafView &lv, int coded, uint64_t n, uint64_t E, uint32_t G, int p0, bool *tie,
-                             cudaStream_t s)
+                             bool *skip, cudaStream_t s)
 {
     uint64_t root_span = 1;
     for (int l = 0; l < coded; ++l) root_span *= kCodeFan;
-    unsigned long long *d = nullptr, h = 0;
+    unsigned long long *d = nullptr, h[2] = {0, 0};
     cudaError_t e = cudaMalloc(&d, sizeof(h));
     if (e != cudaSuccess) return e;
     e = cudaMemsetAsync(d, 0, sizeof(h), s);
     if (e == cudaSuccess) {
-        k_walk_ties<K><<<fill_grid(E), 256, 0, s>>>(lv, root_span, n, E, G, p0, d);
+        if (coded) k_walk_ties<K><<<fill_grid(E), 256, 0, s>>>(lv, root_span, n, E, G, p0, d);
+        if constexpr (sizeof(K) > 8) k_walk_runs<<<fill_grid(n), 256, 0, s>>>(lv, n, p0, d + 1);
         e = cudaGetLastError();
     }
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&h, d, sizeof(h), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(h, d, sizeof(h), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     cudaFree(d);
-    *tie = h > E / 256;
+    *tie = h[0] > E / 256;
+    *skip = h[1] > 16 * n;
     return e;
 }
 
@@ -260,17 +289,18 @@ cudaError_t walk_build(bt_tree *t, const void *h_keys, cudaStream_t s)
     // none where codes tie; then levels of full words down to walk_max_segs
     // (without codes half of it)
     uint64_t segs = E, span = 1, count[kWalkLevels];
-    if (E > kWalkSegs) {
-        w.coded = (E + kCodeFan - 1) / kCodeFan <= kWalkSegs ? 1 : 2;
-        bool tie = false;
-        e = kb == 32 ? codes_tie<Key32>(lv, w.coded, n, E, G, w.p0, &tie, s)
-            : kb == 8 ? codes_tie<uint64_t>(lv, w.coded, n, E, G, w.p0, &tie, s)
-                      : codes_tie<uint32_t>(lv, w.coded, n, E, G, w.p0, &tie, s);
+    if (E > kWalkSegs) w.coded = (E + kCodeFan - 1) / kCodeFan <= kWalkSegs ? 1 : 2;
+    if (w.coded || kb == 32) {
+        bool tie = false, skip = false;
+        e = kb == 32 ? codes_tie<Key32>(lv, w.coded, n, E, G, w.p0, &tie, &skip, s)
+            : kb == 8 ? codes_tie<uint64_t>(lv, w.coded, n, E, G, w.p0, &tie, &skip, s)
+                      : codes_tie<uint32_t>(lv, w.coded, n, E, G, w.p0, &tie, &skip, s);
         if (e == cudaErrorMemoryAllocation) {
             cudaGetLastError();  // no room for an index then
             return cudaSuccess;
         }
         if (e != cudaSuccess) return e;
+        if (skip) return cudaSuccess;
         if (tie) w.coded = 0;
     }
     for (int l = 0; l < w.coded; ++l) {

@@ -43,7 +43,8 @@
 // 32-byte keys are walked by one 64-bit word, the 8 bytes after the bytes all
 // keys share: a query between the smallest and the largest key shares those
 // bytes too, so the word orders it among the keys up to ties, and the entry
-// found is the first whose word is not below the query's.
+// found is the first whose word is not below the query's.  A tree whose words
+// tie in long runs gets no walk index.
 #pragma once
 
 #include <cuda_runtime.h>

@@ -95,10 +95,11 @@ def test_keys_that_crowd(bt, kind, kw, n):
 
 
 @pytest.mark.parametrize("n", [1, 2, 4096, 4097, 17 * 4096 + 1])
-@pytest.mark.parametrize("tie", [0, 7, 5000])
+@pytest.mark.parametrize("tie", [0, 7, 100, 5000])
 def test_byte_keys_with_tied_words(bt, n, tie):
     """Runs of `tie` keys that share the 8 bytes the index walks and differ
-    only later, so that the search has to go on from the first of a run;
+    only later, so that the search has to go on from the first of a run (at
+    5000 keys to a run the tree has no index and descends);
     queries inside runs, at their ends, between them and outside all keys."""
     g = W.rng(910 + n + tie)
     keys = g.integers(0, 256, size=(n, 32), dtype=np.uint8)
@@ -220,3 +221,33 @@ def test_host_buffers_in_place_and_copied(bt, kw, vw, where):
     ov, of = o.search(q)[:2]
     got = hv[: nq * vw // 8].numpy().copy().view(np.uint64 if vw == 64 else np.uint32)
     assert np.array_equal(got.astype(np.uint64), ov) and np.array_equal(hf.numpy(), of)
+
+
+def test_walk_and_host_buffers_under_capture(bt):
+    """A search and one from page-locked host buffers captured in one graph;
+    the replay reads what the buffers hold then."""
+    import torch
+    keys = W.uniform_keys(300_000, 64, seed=950)
+    vals = W.rank_values(keys.size, 64)
+    tree = bt.BTree(keys, vals, 32)
+    o = OracleTree(keys, vals, 32)
+    nq = 40_013
+    dq = torch.zeros(nq, dtype=torch.int64, device="cuda")
+    hq = torch.zeros(nq, dtype=torch.int64, pin_memory=True)
+    v, f = tree.alloc_outputs(nq)
+    hv, hf = torch.zeros(nq, dtype=torch.int64, pin_memory=True), torch.zeros(nq, dtype=torch.uint8, pin_memory=True)
+    ws, nb = tree.alloc_workspace(nq, host=True)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        bt.bt_search_batch(tree.handle, dq, nq, v, f, ws, nb)
+        bt.bt_search_batch_host(tree.handle, hq, nq, hv, hf, ws, nb)
+    for seed in (951, 952):
+        q = [W.make_queries(keys, nq, 0.8, seed=seed + k, width_bits=64) for k in (0, 10)]
+        dq.copy_(torch.from_numpy(q[0].view(np.int64)))
+        hq.copy_(torch.from_numpy(q[1].view(np.int64)))
+        graph.replay()
+        torch.cuda.synchronize()
+        for gv, gf, qq in ((v.cpu().numpy(), f.cpu().numpy(), q[0]), (hv.numpy().view(np.uint64), hf.numpy(), q[1])):
+            ov, of = o.search(qq)[:2]
+            assert np.array_equal(gv, ov) and np.array_equal(gf, of)
