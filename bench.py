@@ -49,6 +49,9 @@ L2_FLUSH_BYTES = 256 << 20
 # from one ncu capture of it (summarised under profiles/); valid only while
 # the descent's source (desc_pipe.cu and descent.cuh) hashes to the same value.
 NCU_DESCEND_TRAFFIC = {"descend_src_sha256": "9f8dc9871dc2dfda", "bytes_per_launch": 223253760}
+# The same for the walk (k_walk) of the default workload.
+WALK_SRC = ("walk.cu", "walk.cuh")
+NCU_WALK_TRAFFIC = {"walk_src_sha256": "8c2f6cb4e5c96725", "bytes_per_launch": 149225984}
 
 
 def parse_args(argv=None):
@@ -281,11 +284,11 @@ class ClockSampler:
                 "reasons": sorted(reasons), "samples": len(self.samples)}
 
 
-def src_sha256() -> str:
-    """Hash of the descent's source: the pipelined kernel's file and the
-    helpers it includes."""
+def src_sha256(names=("desc_pipe.cu", "descent.cuh")) -> str:
+    """Hash of a kernel's source: its file and the helpers it includes (the
+    pipelined descent's unless others are named)."""
     h = hashlib.sha256()
-    for name in ("desc_pipe.cu", "descent.cuh"):
+    for name in names:
         with open(os.path.join(ROOT, "paper_2604_21117_gb300", "csrc", name), "rb") as f:
             h.update(f.read())
     return h.hexdigest()[:16]
@@ -381,27 +384,38 @@ def cpu_baseline(keys, vals, m, q, repeats: int = 100):
                        "untimed; value = all cores")}
 
 
+def walk_algorithmic_bytes(keys, q, kb: int, vb: int) -> float:
+    """Bytes a walk of the batch as given cannot do without: every query and
+    result once, and every distinct one-sector entry the batch reaches (an
+    entry holds 32 / (kb + vb) consecutive keys with their values)."""
+    group = 32 // (kb + vb)
+    entries = np.unique(np.minimum(np.searchsorted(keys, q), keys.size - 1) // group).size
+    return float(q.size * (kb + vb + 1) + 32 * entries)
+
+
 # ------------------------------------------------------ designs leg
 
 DESIGNS = (
-    ("pipelined, inner staged, binary search, L2 window", dict(staging=2, inner=1, ballot=0, l2=64 << 20, lq=1)),
+    # the default: the batch as given through the walk index
+    ("walk index: the batch as given", dict(staging=2, inner=2, ballot=0, l2=0, lq=1, sort_bits=0)),
+    ("pipelined, inner staged, binary search, L2 window", dict(staging=2, inner=1, ballot=0, l2=64 << 20, lq=1,
+                                                               sort_bits=20)),
     ("pipelined, inner staged, ballot + popc, L2 window", dict(staging=2, inner=1, ballot=1, l2=64 << 20, lq=1)),
-    ("pipelined, inner through L1, binary search, L2 window", dict(staging=2, inner=0, ballot=0, l2=64 << 20, lq=1)),
-    ("pipelined, inner staged, binary search, no L2 window", dict(staging=2, inner=1, ballot=0, l2=0, lq=1)),
+    ("pipelined, inner through L1, binary search, L2 window", dict(staging=2, inner=0, ballot=0, l2=64 << 20, lq=1,
+                                                                   sort_bits=20)),
+    ("pipelined, inner staged, binary search, no L2 window", dict(staging=2, inner=1, ballot=0, l2=0, lq=1,
+                                                                  sort_bits=20)),
     ("synchronous cp.async (every level staged, waited)", dict(staging=0, inner=0, ballot=0, l2=0, lq=1)),
     ("synchronous bulk copy", dict(staging=1, inner=0, ballot=0, l2=0, lq=1)),
     ("synchronous, two queries per lane", dict(staging=0, inner=0, ballot=0, l2=0, lq=2)),
-    # not the paper's method: no sort, each warp takes 32 queries as they come
-    ("no sort: the batch as given, pipelined, inner through L1", dict(staging=2, inner=0, ballot=0, l2=64 << 20,
-                                                                      lq=1, sort_bits=0)),
 )
 
 
 def designs_leg(a, bt, tree, dq, out_v, out_f, ws, nb, stream, alg, pool, steps: int = 40):
-    """A/B of the descent designs on the same batches (sorted, except the
-    design that skips the sort): mean descent and step time (CUDA events),
-    and the descent's achieved GB/s of the sorted batch's algorithmic bytes;
-    each design's results are checked against the default design's on the
+    """A/B of the walk and the descent designs on the same batches: mean
+    descent (walk) and step time (CUDA events), and achieved GB/s of the
+    descent's algorithmic bytes, which the walk does not move (none reported
+    for it); each design's results are checked against the default's on the
     last batch."""
     import torch
     B = a.batch
@@ -428,7 +442,7 @@ def designs_leg(a, bt, tree, dq, out_v, out_f, ws, nb, stream, alg, pool, steps:
         desc = [e[1].elapsed_time(e[2]) for e in ev]
         step = [e[0].elapsed_time(e[2]) for e in ev]
         byts = statistics.fmean(alg[i % pool][2] for i in range(steps))
-        gbs = byts / (statistics.fmean(desc) / 1e3) / 1e9
+        gbs = byts / (statistics.fmean(desc) / 1e3) / 1e9 if sb != 0 else None
         v = out_v.cpu().numpy()
         f = out_f.cpu().numpy()
         if ref_v is None:
@@ -436,7 +450,7 @@ def designs_leg(a, bt, tree, dq, out_v, out_f, ws, nb, stream, alg, pool, steps:
         else:
             same = bool(np.array_equal(v, ref_v) and np.array_equal(f, ref_f))
         out[label] = {"descend_us": 1e3 * statistics.fmean(desc), "step_us": 1e3 * statistics.fmean(step),
-                      "descend_gbs": gbs, "descend_frac_of_peak": gbs / peak, "same_results": same}
+                      "descend_gbs": gbs, "descend_frac_of_peak": gbs / peak if gbs else None, "same_results": same}
     bt.bt_tree_set_staging(tree.handle, a.staging)
     bt.bt_tree_set_lane_queries(tree.handle, a.lane_queries)
     bt.bt_tree_set_descent(tree.handle, a.inner, a.ballot)
@@ -845,7 +859,7 @@ def batching_leg(a, bt, stream, nbatches: int = 10_000):
                             "staging": int(ft.staging), "sample_us": float(ft.us), "tune_s": ftune_s,
                             "sample": "1000 batches of the same mix, another seed"},
             "graph_launch": {"lookups_per_s": total / (statistics.fmean(us) / 1e6), "p50_us": us[len(us) // 2],
-                             "p99_us": us[min(len(us) - 1, int(0.99 * len(us)))], "launches_per_work_list": 2},
+                             "p99_us": us[min(len(us) - 1, int(0.99 * len(us)))], "launches_per_work_list": 1},
             "graph_launch_tree_settings": {"lookups_per_s": total / (statistics.fmean(us_tree) / 1e6),
                                            "p50_us": us_tree[len(us_tree) // 2]},
             "per_batch_launches": {"lookups_per_s": total / (per_batch_us / 1e6), "device_us": per_batch_us,
@@ -1105,22 +1119,29 @@ def run_ours(a):
     hit = (pos < keys.size) & (keys[np.minimum(pos, keys.size - 1)] == last)
     ok = bool(np.array_equal(got_f.astype(bool), hit) and np.array_equal(got_v[hit], vals[pos[hit]]))
 
-    # bytes and roofline of the dominant kernel (the descent)
-    desc_bytes = [alg[i % pool][2] for i in range(K)]
+    # bytes and roofline of the dominant kernel: the walk, or where the batch
+    # is partitioned the descent
+    walk = sort_bits <= 0 and a.staging == 2 and a.lane_queries == 1 and a.ballot == 0
+    walk_bytes = [walk_algorithmic_bytes(keys, qb, kb, vb) for qb in batches] if walk else None
+    desc_bytes = [walk_bytes[i % pool] if walk else alg[i % pool][2] for i in range(K)]
     node_bytes = [sum(alg[i % pool][0]) * m * kb + alg[i % pool][1] * 32 for i in range(K)]
     achieved = statistics.fmean(desc_bytes) / (statistics.fmean(desc_ms) / 1e3) / 1e9
     peak, peak_kind = measured_peaks()
     traffic = None
     default_workload = (a.keys == 1 << 24 and a.batch == 1 << 20 and a.fanout == 32 and a.zipf is None
                         and abs(a.hit - 0.9) < 1e-9)
-    if (NCU_DESCEND_TRAFFIC["descend_src_sha256"] == src_sha256() and default_workload and a.lane_queries == 1
+    if walk:
+        if NCU_WALK_TRAFFIC["walk_src_sha256"] == src_sha256(WALK_SRC) and default_workload:
+            traffic = NCU_WALK_TRAFFIC["bytes_per_launch"]
+    elif (NCU_DESCEND_TRAFFIC["descend_src_sha256"] == src_sha256() and default_workload and a.lane_queries == 1
             and a.staging == 2 and a.inner in (1, 2) and a.ballot == 0 and a.l2_window == 64 << 20 and a.warps <= 0
-            and a.pin < 0 and a.sort_bits < 0):
+            and a.pin < 0):
         traffic = NCU_DESCEND_TRAFFIC["bytes_per_launch"]
     step_gbs = statistics.fmean(node_bytes) / (total_s / K) / 1e9  # per batch, at the whole job's rate
+    step_bytes = desc_bytes if walk else node_bytes
+    job_gbs = statistics.fmean(step_bytes) / (total_s / K) / 1e9
     # our kernels per step: one walk of the batch as given, or the partition's
     # kernels and the descent
-    walk = sort_bits <= 0 and a.staging == 2 and a.lane_queries == 1 and a.ballot == 0
     launches_per_step = 1 if walk else bt.bt_sort_launches(tree.handle, B, sort_bits) + 1
     sdev = sorted(step_ms)
 
@@ -1155,19 +1176,28 @@ def run_ours(a):
                      "step_with_phase_event": statistics.fmean(phase_step_ms),
                      "note": "one stream, launch shapes uncapped, an event between the phases (which keeps "
                              "the descent from starting under the partition's tail)"},
-        "hbm_gbs": step_gbs,
-        "roofline": {"kernel": "k_descend (level-wise descent + leaf probe + scatter)", "bound": "hbm",
+        "hbm_gbs": job_gbs,
+        "roofline": {"kernel": ("k_walk (the batch as given through the walk index)" if walk else
+                                "k_descend (level-wise descent + leaf probe + scatter)"),
+                     "bound": "divergent one-sector reads (L1), random memory accesses" if walk else "hbm",
                      "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                      "peak_kind": f"{peak_kind} (hbm_gbs)", "traffic": traffic,
                      "algorithmic_bytes_per_launch": statistics.fmean(desc_bytes),
                      "distinct_nodes_per_level": alg[0][0], "distinct_value_sectors": alg[0][1],
-                     # the whole search per batch (sort + descent): bytes of the distinct
-                     # nodes the batch touches (and its value sectors) over the step time
-                     "per_batch": {"what": "distinct node bytes + value sectors per batch / (whole job time / steps)",
-                                   "bytes": statistics.fmean(node_bytes), "achieved": step_gbs,
-                                   "frac": step_gbs / peak},
-                     "target": {"frac": 0.5, "applies_to": "per_batch (the whole search, sort included)",
-                                "met": step_gbs / peak >= 0.5, "descent_kernel_alone_met": achieved / peak >= 0.5}},
+                     # the whole search per batch over the whole job's time: the bytes the
+                     # path cannot do without
+                     "per_batch": {"what": ("queries, results and distinct entries per batch" if walk else
+                                            "distinct node bytes + value sectors per batch")
+                                   + " / (whole job time / steps)",
+                                   "bytes": statistics.fmean(step_bytes), "achieved": job_gbs,
+                                   "frac": job_gbs / peak},
+                     # what the level-wise descent would have to move for the same batch
+                     # (distinct nodes and value sectors), over the same time
+                     "level_wise_equivalent": {"bytes": statistics.fmean(node_bytes), "gbs": step_gbs,
+                                               "frac": step_gbs / peak},
+                     "target": {"frac": 0.5, "applies_to": "per_batch (the whole search)",
+                                "met": job_gbs / peak >= 0.5,
+                                "level_wise_equivalent_met": step_gbs / peak >= 0.5}},
         "gpu_launches": launches_per_step * K,
         "correct_last_step": ok, "wall_s_timed_loop": wall,
     }
