@@ -51,7 +51,7 @@ L2_FLUSH_BYTES = 256 << 20
 NCU_DESCEND_TRAFFIC = {"descend_src_sha256": "9f8dc9871dc2dfda", "bytes_per_launch": 223253760}
 # The same for the walk (k_walk) of the default workload.
 WALK_SRC = ("walk.cu", "walk.cuh")
-NCU_WALK_TRAFFIC = {"walk_src_sha256": "8c2f6cb4e5c96725", "bytes_per_launch": 149225984}
+NCU_WALK_TRAFFIC = {"walk_src_sha256": "046c7cf09acd3f7f", "bytes_per_launch": 149225984}
 
 
 def parse_args(argv=None):

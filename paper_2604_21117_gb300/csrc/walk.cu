@@ -12,6 +12,8 @@ namespace btgb {
 
 // --------------------------------------------------------- construction
 
+constexpr uint64_t kWalkAskBytes = 32ull << 20;  // larger indexes are held to a share of the free memory
+
 // Where the key of rank i lies in the tree image's leaves.
 struct LeafView {
     const void *keys, *vals;
@@ -337,10 +339,15 @@ cudaError_t walk_build(bt_tree *t, const void *h_keys, cudaStream_t s)
     bytes = (bytes + 255) & ~255ull;
     const uint64_t ent_off = bytes;
     bytes += E * walk_entry_bytes(kb);
-    size_t free_b = 0, total_b = 0;
-    e = cudaMemGetInfo(&free_b, &total_b);
-    if (e != cudaSuccess) return e;
-    if (bytes > free_b / 4) return cudaSuccess;
+    // At most a quarter of what is free.  Only a large index asks how much
+    // that is: the answer takes 18 us (bt_build of 1000 uint64 keys: 182 us
+    // with it, 163 without; 140 with no index).
+    if (bytes > kWalkAskBytes) {
+        size_t free_b = 0, total_b = 0;
+        e = cudaMemGetInfo(&free_b, &total_b);
+        if (e != cudaSuccess) return e;
+        if (bytes > free_b / 4) return cudaSuccess;
+    }
     e = cudaMalloc(&t->d_walk, bytes);
     if (e == cudaErrorMemoryAllocation) {
         cudaGetLastError();  // searched by the descent, as without this index
