@@ -128,6 +128,7 @@ struct bt_tree {
     void *d_paper;
     btgb::WalkDev walk;  // valid while d_walk is set
     void *d_walk;        // the walk index (null: not built)
+    bool walk_own;       // it is an allocation of its own, not part of the image's
 };
 
 struct bt_model {

@@ -486,7 +486,14 @@ extern "C" bt_status bt_build(const void *h_keys, const void *h_vals, uint64_t n
         node_max.swap(upper_max);
     }
 
-    cudaError_t e = cudaMalloc(&t->d_image, off);
+    // a small tree's walk index lies behind the image
+    uint64_t room = walk_room(n, kb, vb);
+    cudaError_t e = cudaMalloc(&t->d_image, off + room);
+    if (e == cudaErrorMemoryAllocation && room) {
+        cudaGetLastError();
+        room = 0;
+        e = cudaMalloc(&t->d_image, off);
+    }
     if (e != cudaSuccess) {
         set_error_detail("cudaMalloc(tree image)", e);
         free(img);
@@ -511,7 +518,7 @@ extern "C" bt_status bt_build(const void *h_keys, const void *h_vals, uint64_t n
     d.split_off = kb == 32 ? static_cast<unsigned char *>(t->d_image) + split_off_offset : nullptr;
     d.split_R = reinterpret_cast<const uint16_t *>(static_cast<unsigned char *>(t->d_image) + split_R_offset);
     t->info.d_image = t->d_image;
-    e = walk_build(t, h_keys, s);
+    e = walk_build(t, h_keys, room ? static_cast<unsigned char *>(t->d_image) + off : nullptr, room, s);
     if (e != cudaSuccess) {
         set_error_detail("walk index", e);
         bt_free(t);
@@ -524,7 +531,7 @@ extern "C" bt_status bt_build(const void *h_keys, const void *h_vals, uint64_t n
 extern "C" void bt_free(bt_tree *t)
 {
     if (!t) return;
-    if (t->d_walk) cudaFree(t->d_walk);
+    if (t->d_walk && t->walk_own) cudaFree(t->d_walk);
     if (t->d_image) cudaFree(t->d_image);
     if (t->d_paper) cudaFree(t->d_paper);
     delete t;

@@ -375,11 +375,15 @@ cudaError_t descend_paper_layout(const DevTree &t, const PaperTree &p, const voi
                                  const void *recs, uint64_t nq, void *out_v, uint8_t *out_f, cudaStream_t s);
 
 // Builds the walk index of a tree whose image is on the device (h_keys: the
-// sorted keys it was built from), in an allocation of its own.  Leaves the tree without one (and returns
+// sorted keys it was built from), in the `room` bytes at d_room where they
+// suffice, else in an allocation of its own.  Leaves the tree without one (and returns
 // cudaSuccess) when the index would take more than a quarter of the free
 // device memory, the key count exceeds what its node numbers hold, or
 // 32-byte keys share the words it walks in long runs.
-cudaError_t walk_build(bt_tree *tree, const void *h_keys, cudaStream_t s);
+cudaError_t walk_build(bt_tree *tree, const void *h_keys, unsigned char *d_room, uint64_t room, cudaStream_t s);
+// Bytes behind the image of a tree of n keys that hold its walk index, 0 for
+// trees whose index is large.
+uint64_t walk_room(uint64_t n, int key_bytes, int val_bytes);
 // Search of a batch as given through the walk index; md: with a model of the
 // tree (integer keys).
 cudaError_t walk_search(const bt_tree *tree, const void *q, uint64_t nq, void *out_v, uint8_t *out_f, cudaStream_t s,
