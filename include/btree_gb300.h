@@ -130,13 +130,13 @@ typedef struct bt_info {
  * bits above the smallest key are below j (32-byte keys: bits of the 8 bytes
  * after the bytes all keys share).
  *
- * Beside the image, in an allocation of its own that bt_info does not count,
- * the device keeps a walk index: the keys and values once more in one-sector
+ * Behind the image (up to 8 MB of entries), or in an allocation of its own,
+ * and not counted by bt_info, the device keeps a walk index: the keys and values once more in one-sector
  * entries (32-byte keys: 64 bytes each) under one-sector nodes, through which
  * batches are searched as given (see bt_search_opts.sort_bits).  It takes
  * about 18 bytes per 64-bit key and value (9 for 32-bit ones, 66 per 32-byte
  * key), more where keys crowd (up to 20, 10 and 72), and is left out when
- * that is more than a quarter of the free device memory, or where the 8 bytes
+ * that is above 32 MB and more than a quarter of the free device memory, or where the 8 bytes
  * after the bytes all 32-byte keys share are the same for hundreds of keys on
  * end; searches are then partitioned and descend the tree as bt_sort_bits
  * says.
