@@ -51,7 +51,7 @@ L2_FLUSH_BYTES = 256 << 20
 NCU_DESCEND_TRAFFIC = {"descend_src_sha256": "9f8dc9871dc2dfda", "bytes_per_launch": 223253760}
 # The same for the walk (k_walk) of the default workload.
 WALK_SRC = ("walk.cu", "walk.cuh")
-NCU_WALK_TRAFFIC = {"walk_src_sha256": "6855d6fd5c6a689f", "bytes_per_launch": 149225984}
+NCU_WALK_TRAFFIC = {"walk_src_sha256": "7be9d83980805df0", "bytes_per_launch": 149225984}
 
 
 def parse_args(argv=None):

