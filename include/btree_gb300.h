@@ -545,13 +545,15 @@ bt_status bt_tree_set_l2_window(bt_tree *tree, uint64_t max_bytes);
  * the paper's kernel.  BT_ERR_ARG above 32. */
 bt_status bt_tree_set_corun(bt_tree *tree, uint32_t descent_blocks_per_sm, uint32_t partition_blocks_per_sm);
 
-/* Test hook: poll limit of the first bounded wait of the descents' bulk-copy
- * staging, BT_DEFAULT_WAIT_POLLS unless changed; 0 makes every such wait
- * give up at once.  After a wait gives up, the warp counts it
- * (bt_check_timeouts then returns BT_ERR_TIMEOUT), waits once more with the
- * default limit so that its copies land, and stops: the outputs of that
- * search are invalid.  Process-wide; takes effect for launches made after
- * the call.  No counterpart in the paper. */
+/* Test hook: poll limit of the first bounded wait for bulk copies of a search
+ * (a descent's staging, the walk index's top), BT_DEFAULT_WAIT_POLLS unless
+ * changed; 0 makes every such wait give up at once.  After a wait gives up,
+ * the warp counts it (bt_check_timeouts then returns BT_ERR_TIMEOUT), waits
+ * once more with the default limit so that its copies land, and stops: the
+ * outputs of that search are invalid.  In a work list that goes through the
+ * walk indexes (bt_forest_search, the server) the warp does not stop but reads
+ * the tops from device memory: those outputs are valid.  Process-wide; takes
+ * effect for launches made after the call.  No counterpart in the paper. */
 #define BT_DEFAULT_WAIT_POLLS (1u << 22)
 void bt_debug_set_wait_polls(uint32_t polls);
 
@@ -564,8 +566,8 @@ void bt_debug_set_wait_polls(uint32_t polls);
 bt_status bt_tree_set_lane_queries(bt_tree *tree, uint32_t per_lane);
 
 /* BT_ERR_TIMEOUT if a bounded device wait of a search gave up since the
- * last call (the results of such a search are invalid), else BT_OK; clears
- * the counters.  Synchronous (reads device counters).  No counterpart in the
+ * last call (the results of such a search are invalid, those of a work list
+ * excepted: see bt_debug_set_wait_polls), else BT_OK; clears the counters.  Synchronous (reads device counters).  No counterpart in the
  * paper (its kernel has no waits that can fail). */
 bt_status bt_check_timeouts(void);
 

@@ -65,7 +65,7 @@ __global__ void __launch_bounds__(kWalkForestThreads)
     k_forest_walk(const ForestWalk *__restrict__ gtab, uint32_t ntrees, uint32_t top_total,
                   const bt_batch_desc *__restrict__ batches, uint32_t nb, const uint32_t *__restrict__ chunk_start,
                   const K *__restrict__ q, uint64_t nq, V *__restrict__ out_v, uint8_t *__restrict__ out_f,
-                  ForestDone done)
+                  ForestDone done, uint32_t wait_polls)
 {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ __align__(8) uint64_t bar;
@@ -123,10 +123,13 @@ __global__ void __launch_bounds__(kWalkForestThreads)
         if (threadIdx.x == blockDim.x - 1) rows[nrows] = run;
     }
     __syncthreads();
-    bool ok = true;
-    if (top_total && !mbar_wait_warp(&bar, 0, kMbarSpinLimit)) {
+    // A warp whose wait gives up is counted and reads every top through L1, as
+    // those without a place: the completion signal below says that the whole
+    // list has been searched, and whoever polls it reads no other word.
+    bool tops_here = true;
+    if (top_total && !mbar_wait_warp(&bar, 0, wait_polls)) {
         mbar_give_up(&bar, 0, static_cast<int>(lane));
-        ok = false;
+        tops_here = false;
     }
     auto row_pos = [&](uint32_t r) -> uint64_t { return unit ? chunk_start[r * 32] : rows[r]; };
     const uint64_t total = unit ? chunk_start[nb] : rows[nrows];
@@ -135,7 +138,7 @@ __global__ void __launch_bounds__(kWalkForestThreads)
     const uint64_t b0 = total / gridDim.x * blockIdx.x + total % gridDim.x * blockIdx.x / gridDim.x;
     const uint64_t b1 = total / gridDim.x * (blockIdx.x + 1) + total % gridDim.x * (blockIdx.x + 1) / gridDim.x;
     const uint64_t p = b0 + (b1 - b0) * warp / nw, p1 = b0 + (b1 - b0) * (warp + 1) / nw;
-    if (ok && p < p1) {
+    if (p < p1) {
         uint32_t lo = 0, hi = nrows - 1;  // the last row that starts at or before p
         while (lo < hi) {
             const uint32_t mid = (lo + hi + 1) / 2;
@@ -223,7 +226,7 @@ __global__ void __launch_bounds__(kWalkForestThreads)
             if (F.w.n) {
                 // (two calls, so that each reads the top by its own address space)
                 uint32_t entry;
-                if (F.top_off != kNoTop) {
+                if (tops_here && F.top_off != kNoTop) {
                     const unsigned char *top = smem + F.top_off;
                     entry = walk_entry<K>(F.w, top, walk_segment<K>(F.w, top, now.key), now.key);
                 } else {
@@ -287,7 +290,7 @@ static cudaError_t walk_forest_launch(const ForestWalk *tab, uint32_t ntrees, ui
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kern, tab, ntrees, top_total, b, nb, cs, static_cast<const K *>(q), nq,
-                              static_cast<V *>(ov), of, done);
+                              static_cast<V *>(ov), of, done, first_wait_polls());
 }
 
 cudaError_t forest_walk_run(const ForestWalk *tab, uint32_t ntrees, uint32_t top_total, int kb, int vb,

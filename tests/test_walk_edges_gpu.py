@@ -1,0 +1,91 @@
+"""Edges of the searches through the walk index: waits that run out, buffers
+that overlap or are page-locked in part, and trees at the sizes where the
+index changes shape."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+from oracle import OracleTree
+from paper_2604_21117_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def bt():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2604_21117_gb300 import build_lib
+    build_lib.build()
+    from paper_2604_21117_gb300 import btree
+    return btree
+
+
+def _dev(a):
+    import torch
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+@pytest.fixture
+def no_polls(bt):
+    """Every bounded wait gives up at once while the test runs."""
+    import torch
+    torch.cuda.synchronize()
+    bt.bt_check_timeouts()  # clear anything earlier
+    bt.bt_debug_set_wait_polls(0)
+    yield
+    torch.cuda.synchronize()
+    bt.bt_debug_set_wait_polls(bt.BT_DEFAULT_WAIT_POLLS)
+
+
+def _two_trees(bt):
+    out = []
+    for i, n in enumerate((20_000, 300_000)):
+        keys = W.uniform_keys(n, 64, seed=960 + i)
+        vals = W.rank_values(n, 64)
+        out.append((keys, bt.BTree(keys, vals, 32), OracleTree(keys, vals, 32)))
+    return out
+
+
+def test_work_list_whose_wait_gives_up_is_searched_all_the_same(bt, no_polls):
+    """The wait for the tops gives up in every warp: reported, and every
+    result is there (a completion flag says that the list has been searched)."""
+    import torch
+    trees = _two_trees(bt)
+    forest = bt.bt_forest_create([t[1].handle for t in trees])
+    nb, per = 300, 77
+    desc = np.zeros(nb, bt.BATCH_DESC_DTYPE)
+    desc["tree"], desc["count"], desc["offset"] = np.arange(nb) % 2, per, np.arange(nb) * per
+    q = np.concatenate([W.make_queries(trees[i % 2][0], per, 0.8, seed=970 + i, width_bits=64) for i in range(nb)])
+    v = torch.full((nb * per,), 5, dtype=torch.int64, device="cuda")
+    f = torch.full((nb * per,), 9, dtype=torch.uint8, device="cuda")
+    wsb = bt.bt_forest_workspace_bytes(nb)
+    ws = torch.empty(wsb, dtype=torch.uint8, device="cuda")
+    bt.bt_forest_search(forest, _dev(desc.view(np.uint8)), nb, _dev(q), v, f, ws, wsb)
+    with pytest.raises(bt.BTreeError) as e:
+        bt.bt_check_timeouts()
+    assert e.value.code == "BT_ERR_TIMEOUT"
+    gv, gf = v.cpu().numpy().view(np.uint64).reshape(nb, per), f.cpu().numpy().reshape(nb, per)
+    for i in range(2):
+        ov, of = trees[i][2].search(q.reshape(nb, per)[i::2].ravel())[:2]
+        assert np.array_equal(gv[i::2].ravel(), ov) and np.array_equal(gf[i::2].ravel(), of)
+    bt.bt_forest_free(forest)
+
+
+def test_served_requests_have_their_results_when_waits_give_up(bt, no_polls):
+    trees = _two_trees(bt)
+    srv = bt.bt_server_create([t[1] for t in trees], None, slots=2, max_batch=512, deadline_us=20.0)
+    for r in range(40):
+        q = W.make_queries(trees[r % 2][0], 1 + 9 * r, 0.8, seed=980 + r, width_bits=64)
+        v, f = np.full(q.size, 5, np.uint64), np.full(q.size, 9, np.uint8)
+        ticket = bt.bt_server_submit(srv, r % 2, q, v, f)
+        bt.bt_server_drain(srv, 10.0)
+        assert bt.bt_server_poll(srv, 16) == [ticket]
+        ov, of = trees[r % 2][2].search(q)[:2]
+        assert np.array_equal(v, ov) and np.array_equal(f, of)
+    bt.bt_server_destroy(srv)
+    with pytest.raises(bt.BTreeError) as e:
+        bt.bt_check_timeouts()
+    assert e.value.code == "BT_ERR_TIMEOUT"
