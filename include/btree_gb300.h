@@ -175,7 +175,8 @@ typedef struct bt_search_opts {
      * library choose, 0 skips the partition, 1..21 forces that many bits
      * (larger values mean 21).  A batch that is not forced goes through the
      * tree's walk index as given, the faster way at every size, unless the
-     * tree has none, d_fetch_counts is set, or another descent than the
+     * tree has none, d_fetch_counts is set, its results lie over its queries
+     * (see bt_search_batch), or another descent than the
      * pipelined one with the binary-search rank has been chosen for it
      * (bt_tree_set_staging, bt_tree_set_lane_queries, bt_tree_set_descent);
      * then -1 partitions on bt_sort_bits bits (none below 786432 queries --
@@ -210,7 +211,10 @@ typedef struct bt_search_opts {
  *   ws_bytes     size of d_workspace.
  *
  * Asynchronous on `stream`; allocates nothing, so it may be captured in a
- * CUDA graph.  Queries and outputs must not overlap the workspace.
+ * CUDA graph.  Queries and outputs must not overlap the workspace.  Values as
+ * wide as the keys may be written over the queries, from the same address on;
+ * other results over queries come out right only where bt_sort_bits(tree, nq,
+ * -1) is above 0 (the batch is then partitioned, i.e. copied first).
  * Errors: BT_ERR_ARG, BT_ERR_WORKSPACE, BT_ERR_CUDA.
  */
 bt_status bt_search_batch(const bt_tree *tree, const void *d_queries, uint64_t nq,

@@ -133,13 +133,27 @@ static bool arrays_aligned(const DevTree &t, const void *keys, const void *qidx,
            (reinterpret_cast<uintptr_t>(vals) & (va - 1)) == 0;
 }
 
+// Whether results lie over queries that other warps may not have read yet,
+// when the batch is read where it is.  Values as wide as the keys at the same
+// address do not: the lane that read a query writes its result.
+static bool results_over_queries(const DevTree &t, const void *q, uint64_t nq, const void *vals, const void *found)
+{
+    const uintptr_t q0 = reinterpret_cast<uintptr_t>(q), q1 = q0 + nq * t.key_bytes;
+    auto meets = [&](const void *p, uint64_t bytes) {
+        const uintptr_t r = reinterpret_cast<uintptr_t>(p);
+        return r < q1 && q0 < r + bytes;
+    };
+    return meets(found, nq) || (meets(vals, nq * t.val_bytes) && !(vals == q && t.val_bytes == t.key_bytes));
+}
+
 // Queries per batch from which the automatic choice partitions a batch that
-// does not go through the walk index, for trees larger than a quarter of the L2 (DevTree::sort_pays).  Measured
-// on uint64 trees at fanout 32: on 2^24 keys the unsorted descent is faster
-// up to 2^19 queries (53 against 61 us), the sorted search from 2^20 (86
-// against 90 us); on 4 * 10^6 keys (67 MB) likewise (49 against 52 us at 2^19,
-// 79 against 82 at 2^20); on 10^6 keys (17 MB) the unsorted descent is faster
-// at every size to 2^20 (61 against 72 us there).
+// does not go through the walk index, for trees larger than a quarter of the
+// L2 (DevTree::sort_pays).  Measured on uint64 trees at fanout 32: on 2^24
+// keys the unsorted descent is faster up to 2^19 queries (53 against 61 us),
+// the sorted search from 2^20 (86 against 90 us); on 4 * 10^6 keys (67 MB)
+// likewise (49 against 52 us at 2^19, 79 against 82 at 2^20); on 10^6 keys
+// (17 MB) the unsorted descent is faster at every size to 2^20 (61 against 72
+// us there).
 constexpr uint64_t kAutoSortMinBatch = 786432;
 // The same for 32-byte keys, whose comparisons and 512-byte node blocks make
 // the unsorted descent dearer: on 2^20 keys at fanout 16 (47 MB) the sorted
@@ -393,7 +407,12 @@ extern "C" bt_status bt_search_batch_ex(const bt_tree *tree, const void *d_queri
         return BT_OK;
     }
 
-    if (opts ? opts->sort_bits <= 0 && !opts->d_fetch_counts && walk_takes(tree) : walk_takes(tree)) {
+    const PartPlan pp = plan_partition(t, opts ? opts->sort_bits : -1, nq);
+    // (a batch that the automatic choice would partition is copied by that
+    // before any result is written, so its results may lie over it: such a
+    // batch is partitioned still)
+    if ((!opts || (opts->sort_bits <= 0 && !opts->d_fetch_counts)) && walk_takes(tree) &&
+        !(pp.bits > 0 && results_over_queries(t, d_queries, nq, d_out_vals, d_out_found))) {
         e = opts && opts->phase_event ? cudaEventRecord(static_cast<cudaEvent_t>(opts->phase_event), s) : cudaSuccess;
         if (e != cudaSuccess) {
             set_error_detail("phase event", e);
@@ -406,7 +425,6 @@ extern "C" bt_status bt_search_batch_ex(const bt_tree *tree, const void *d_queri
         }
         return BT_OK;
     }
-    const PartPlan pp = plan_partition(t, opts ? opts->sort_bits : -1, nq);
     const void *q = d_queries;
     const uint32_t *qidx = nullptr;
     const void *recs = nullptr;
@@ -639,7 +657,9 @@ extern "C" bt_status bt_learned_search_batch(const bt_tree *tree, const bt_model
     if (!d_workspace || ws_bytes < w.total || (reinterpret_cast<uintptr_t>(d_workspace) & 255u))
         return BT_ERR_WORKSPACE;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    if (tree->d_walk) {
+    const PartPlan pp = plan_partition(t, -1, nq);
+    // (results over a batch that would be partitioned: as in bt_search_batch_ex)
+    if (tree->d_walk && !(pp.bits > 0 && results_over_queries(t, d_queries, nq, d_out_vals, d_out_found))) {
         const cudaError_t we = walk_search(tree, d_queries, nq, d_out_vals, d_out_found, s, &model->dev);
         if (we != cudaSuccess) {
             set_error_detail("learned walk launch", we);
@@ -647,7 +667,6 @@ extern "C" bt_status bt_learned_search_batch(const bt_tree *tree, const bt_model
         }
         return BT_OK;
     }
-    const PartPlan pp = plan_partition(t, -1, nq);
     const void *q = d_queries;
     const uint32_t *qidx = nullptr;
     const void *recs = nullptr;

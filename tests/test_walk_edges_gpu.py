@@ -89,3 +89,35 @@ def test_served_requests_have_their_results_when_waits_give_up(bt, no_polls):
     with pytest.raises(bt.BTreeError) as e:
         bt.bt_check_timeouts()
     assert e.value.code == "BT_ERR_TIMEOUT"
+
+
+@pytest.mark.parametrize("learned", [False, True])
+@pytest.mark.parametrize("vw,over", [(32, "values"), (64, "values, 8 bytes on"), (64, "found"), (64, "values, same place")])
+def test_results_over_the_queries_of_a_large_batch(bt, learned, vw, over):
+    """A batch that the automatic choice partitions is copied before results
+    are written: they may lie over the queries, narrower and shifted too."""
+    import torch
+    n, nq = 4_300_000, 800_003
+    keys = W.uniform_keys(n, 64, seed=990)
+    tree = bt.BTree(keys, W.rank_values(n, vw), 32)
+    assert bt.bt_sort_bits(tree.handle, nq) > 0
+    q = W.make_queries(keys, nq, 0.8, seed=991, width_bits=64)
+    pos = np.searchsorted(keys, q)
+    hit = keys[np.minimum(pos, n - 1)] == q
+    want = np.where(hit, pos.astype(np.uint64), np.uint64(2**vw - 1))
+    buf = torch.zeros(8 * nq + 8, dtype=torch.uint8, device="cuda")
+    buf[: 8 * nq] = _dev(q.view(np.uint8))
+    v = torch.zeros(nq * vw // 8, dtype=torch.uint8, device="cuda") if over == "found" else \
+        buf[8 if over.endswith("on") else 0:][: nq * vw // 8]
+    f = buf[5 * nq: 6 * nq] if over == "found" else torch.zeros(nq, dtype=torch.uint8, device="cuda")
+    ws, nb = tree.alloc_workspace(nq)
+    if learned:
+        m = bt.bt_model_train(tree.handle, bt.BT_MODEL_PL, segments=256)
+        bt.bt_learned_search_batch(tree.handle, m, buf.data_ptr(), nq, v, f, ws, nb)
+    else:
+        bt.bt_search_batch(tree.handle, buf.data_ptr(), nq, v, f, ws, nb)
+    got = v.cpu().numpy().view(np.uint64 if vw == 64 else np.uint32).astype(np.uint64)
+    assert np.array_equal(got, want) and np.array_equal(f.cpu().numpy().astype(bool), hit)
+    if learned:
+        bt.bt_model_free(m)
+    tree.close()
