@@ -292,6 +292,9 @@ cudaError_t walk_build(bt_tree *t, const void *h_keys, unsigned char *d_room, ui
     const uint32_t G = walk_group(kb, vb);
     const uint64_t F = walk_fan(kb), E = (n + G - 1) / G;
     if (E >= (1ull << 32)) return cudaSuccess;  // node and entry numbers are 32-bit
+    // what an earlier call left in the runtime (and has reported) is not these
+    // launches' error: before the index a build launched nothing and never asked
+    cudaGetLastError();
     WalkDev w;
     memset(&w, 0, sizeof(w));
     w.n = n;

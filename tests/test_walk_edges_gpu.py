@@ -121,3 +121,25 @@ def test_results_over_the_queries_of_a_large_batch(bt, learned, vw, over):
     if learned:
         bt.bt_model_free(m)
     tree.close()
+
+
+def test_a_reported_error_does_not_fail_the_next_build(bt):
+    """A call refused by the runtime (an allocation while a stream captures)
+    reports its error; the next call starts without it."""
+    import ctypes
+    import torch
+    keys = W.uniform_keys(3000, 64, seed=997)
+    tree = bt.BTree(keys, W.rank_values(3000, 64), 16)
+    cu = ctypes.CDLL("libcuda.so.1")
+    s, graph = torch.cuda.Stream(), ctypes.c_void_p()
+    torch.cuda.synchronize()
+    assert cu.cuStreamBeginCapture_v2(ctypes.c_void_p(s.cuda_stream), 0) == 0  # global: no allocations meanwhile
+    with pytest.raises(bt.BTreeError) as e:
+        bt.bt_forest_create([tree.handle])
+    assert e.value.code == "BT_ERR_CUDA"
+    cu.cuStreamEndCapture(ctypes.c_void_p(s.cuda_stream), ctypes.byref(graph))
+    if graph.value:
+        cu.cuGraphDestroy(graph)
+    again = bt.BTree(keys, W.rank_values(3000, 64), 16)
+    v, f = again.search(_dev(keys))
+    assert np.array_equal(v.cpu().numpy(), np.arange(3000, dtype=np.uint64)) and f.cpu().numpy().all()
