@@ -18,6 +18,7 @@
 //   4. the scatter of each result back to the query's input position.
 // Everything is integer compares; nothing here is a dense contraction, so
 // no tensor-core path is used.
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -469,21 +470,54 @@ extern "C" bt_status bt_search_batch(const bt_tree *tree, const void *d_queries,
                               nullptr, stream);
 }
 
+// Bytes from host address `at` to the end of the page-locked range that holds
+// it, where the GPU sees that range from device address `dev` on; else 0.
+static uint64_t mapped_bytes(uintptr_t at, uintptr_t dev)
+{
+    using Query = CUresult (*)(unsigned, CUpointer_attribute *, void **, CUdeviceptr);
+    static const Query query = [] {
+        void *fn = nullptr;
+        cudaDriverEntryPointQueryResult found = cudaDriverEntryPointSymbolNotFound;
+        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &fn, 7000, cudaEnableDefault, &found) !=
+            cudaSuccess)
+            cudaGetLastError();
+        return found == cudaDriverEntryPointSuccess ? reinterpret_cast<Query>(fn) : nullptr;
+    }();
+    // for an address that is none of CUDA's the query succeeds, all values 0
+    CUmemorytype type = static_cast<CUmemorytype>(0);
+    int managed = 0;
+    CUdeviceptr view = 0, start = 0;
+    size_t size = 0;
+    CUpointer_attribute which[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED,
+                                   CU_POINTER_ATTRIBUTE_DEVICE_POINTER, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
+                                   CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    void *into[] = {&type, &managed, &view, &start, &size};
+    if (!query || query(5, which, into, at) != CUDA_SUCCESS) return 0;
+    if (type != CU_MEMORYTYPE_HOST || managed || view != dev || at < start || at - start >= size) return 0;
+    return size - (at - start);
+}
+
 // The device address of a page-locked host buffer that the GPU can read and
-// write in place, all `bytes` of it and aligned to `align`; else null.
+// write in place, all `bytes` of it and aligned to `align`; else null.  The
+// buffer may lie in a few ranges that were page-locked one after the other.
 static void *mapped_view(const void *h, uint64_t bytes, uint64_t align)
 {
-    cudaPointerAttributes a, b;
-    const unsigned char *last = static_cast<const unsigned char *>(h) + bytes - 1;
-    if (cudaPointerGetAttributes(&a, h) != cudaSuccess || cudaPointerGetAttributes(&b, last) != cudaSuccess) {
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, h) != cudaSuccess) {
         cudaGetLastError();
         return nullptr;
     }
-    if (a.type != cudaMemoryTypeHost || b.type != cudaMemoryTypeHost || !a.devicePointer ||
-        static_cast<unsigned char *>(a.devicePointer) + bytes - 1 != b.devicePointer ||
+    if (a.type != cudaMemoryTypeHost || !a.devicePointer ||
         (reinterpret_cast<uintptr_t>(a.devicePointer) & (align - 1)))
         return nullptr;
-    return a.devicePointer;
+    uint64_t held = 0;
+    for (int range = 0; range < 8 && held < bytes; ++range) {
+        const uint64_t more = mapped_bytes(reinterpret_cast<uintptr_t>(h) + held,
+                                           reinterpret_cast<uintptr_t>(a.devicePointer) + held);
+        if (more == 0) break;
+        held += more;
+    }
+    return held >= bytes ? a.devicePointer : nullptr;
 }
 
 extern "C" bt_status bt_search_batch_host(const bt_tree *tree, const void *h_queries, uint64_t nq,

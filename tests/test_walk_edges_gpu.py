@@ -143,3 +143,63 @@ def test_a_reported_error_does_not_fail_the_next_build(bt):
     again = bt.BTree(keys, W.rank_values(3000, 64), 16)
     v, f = again.search(_dev(keys))
     assert np.array_equal(v.cpu().numpy(), np.arange(3000, dtype=np.uint64)) and f.cpu().numpy().all()
+
+
+
+def _captured_nodes(call, stream):
+    """Nodes of the graph that `call` on the raw stream captures (nothing
+    runs); None when the call fails."""
+    import ctypes
+    cu = ctypes.CDLL("libcuda.so.1")
+    graph, count, s = ctypes.c_void_p(), ctypes.c_size_t(), ctypes.c_void_p(stream)
+    assert cu.cuStreamBeginCapture_v2(s, 2) == 0  # relaxed
+    try:
+        call()
+        failed = False
+    except Exception:
+        failed = True
+    ended = cu.cuStreamEndCapture(s, ctypes.byref(graph))
+    if failed or ended != 0:
+        return None
+    assert cu.cuGraphGetNodes(graph, None, ctypes.byref(count)) == 0
+    assert cu.cuGraphDestroy(graph) == 0
+    return count.value
+
+
+@pytest.mark.parametrize("locked", ["one range", "two ranges", "a gap between two ranges"])
+def test_only_wholly_page_locked_queries_are_read_in_place(bt, locked):
+    """A batch searched in place is one kernel node of a captured graph, one
+    that is copied several (with a gap, only captured: it never runs)."""
+    import mmap
+    import torch
+    part = 1 << 16
+    nq = 3 * part // 8
+    keys = W.uniform_keys(50_000, 64, seed=995)
+    tree = bt.BTree(keys, W.rank_values(keys.size, 64), 32)
+    region = mmap.mmap(-1, 3 * part)
+    q = np.frombuffer(region, np.uint64)
+    q[:] = W.make_queries(keys, nq, 0.8, seed=996, width_bits=64)
+    ranges = {"one range": [(0, 3)], "two ranges": [(0, 1), (1, 2)], "a gap between two ranges": [(0, 1), (2, 1)]}
+    v, f = torch.zeros(nq, dtype=torch.int64, pin_memory=True), torch.zeros(nq, dtype=torch.uint8, pin_memory=True)
+    ws, nb = tree.alloc_workspace(nq, host=True)
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    rt = torch.cuda.cudart()
+    for at, count in ranges[locked]:
+        assert int(rt.cudaHostRegister(q.ctypes.data + at * part, count * part, 0)) == 0
+    try:
+        def call():
+            bt.bt_search_batch_host(tree.handle, q, nq, v, f, ws, nb, stream=stream.cuda_stream)
+        nodes = _captured_nodes(call, stream.cuda_stream)
+        if locked == "a gap between two ranges":
+            assert nodes != 1
+        else:
+            assert nodes == 1
+            call()
+            stream.synchronize()
+            ov, of = OracleTree(keys, W.rank_values(keys.size, 64), 32).search(q.copy())[:2]
+            assert np.array_equal(v.numpy().view(np.uint64), ov) and np.array_equal(f.numpy(), of)
+    finally:
+        torch.cuda.synchronize()
+        for at, _ in ranges[locked]:
+            rt.cudaHostUnregister(q.ctypes.data + at * part)
