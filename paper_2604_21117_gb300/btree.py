@@ -111,19 +111,26 @@ def _check(call: str, st: int):
         raise BTreeError(call, st)
 
 
-# The current stream's raw handle and the current device's number, once torch
-# has CUDA up: torch.cuda.current_stream() builds a Stream object for every
-# call (3.0 of the 7.9 us a small search took to submit; these two take 0.2).
+# What gives the current stream's raw handle from the current device, and the
+# current device, once torch has CUDA up: torch.cuda.current_stream() builds a
+# Stream object for every call (3.0 of the 7.9 us a small search took to
+# submit; these two take 0.2), and is what is asked where torch has them not.
+# _current_device is set last: a thread that finds it set finds both.
 _raw_stream = _current_device = None
 
 
 def _stream_handle(stream) -> int | None:
     global _raw_stream, _current_device
     if stream is None:
-        if _raw_stream is None:
+        if _current_device is None:
             import torch
             handle = torch.cuda.current_stream().cuda_stream
-            _raw_stream, _current_device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+            raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+            device = getattr(torch._C, "_cuda_getDevice", None)
+            if raw is None or device is None:
+                raw, device = (lambda _: torch.cuda.current_stream().cuda_stream), (lambda: 0)
+            _raw_stream = raw
+            _current_device = device
             return handle
         return _raw_stream(_current_device())
     if isinstance(stream, int):
