@@ -451,11 +451,14 @@ bt_status bt_forest_search(const bt_forest *forest, const bt_batch_desc *d_batch
  * bt_forest_autotune -- time the work list (arguments as bt_forest_search)
  * under every combination of warps per block {4, 8, 16}, pin budget
  * {0, 16384, 49152, 98304}, queries per lane {each tree's, 1, 2} and
- * staging {each tree's, all through L1, all staged}; keep the fastest (after 2
- * untimed calls, 3 runs of 5 calls issued back to back behind a short device
- * spin, timed together with CUDA events on `stream`; the median per call) as
- * the forest's settings and return it in *best.  Synchronizes the device.  No counterpart
- * in the paper (its kernel's shape is fixed by the FPGA build).
+ * staging {each tree's, all through L1, all staged} -- the settings under
+ * which the list goes through the walk indexes (bt_forest_create) are one and
+ * the same and timed once, at 8 warps, 16384 bytes and each tree's queries per
+ * lane -- and keep the fastest (after 2 untimed calls, 3 runs of 5 calls
+ * issued back to back behind a short device spin, timed together with CUDA
+ * events on `stream`; the median per call) as the forest's settings and return
+ * it in *best.  Synchronizes the device.  No counterpart in the paper (its
+ * kernel's shape is fixed by the FPGA build).
  * Errors: as bt_forest_search.
  */
 bt_status bt_forest_autotune(bt_forest *forest, const bt_batch_desc *d_batches, uint32_t nbatches,

@@ -743,12 +743,30 @@ extern "C" bt_status bt_forest_autotune(bt_forest *f, const bt_batch_desc *d_bat
     if (e == cudaSuccess) e = cudaEventCreate(&e1);
     const uint32_t warps[] = {4, 8, 16};
     const uint32_t pins[] = {0, 16384, 49152, 98304};
+    // Settings under which the list goes through the walk indexes launch one
+    // and the same kernel (only the staging choice decides that): timed once,
+    // at 8 warps, 16384 pinned bytes and each tree's own queries per lane.
+    constexpr uint32_t kDefaultWarps = 8, kDefaultPin = 16384;
+    bool walks[3] = {false, false, false};
+    for (uint32_t sm = 0; sm <= 2 && e == cudaSuccess; ++sm) {
+        const bt_forest_tune cfg{kDefaultWarps, kDefaultPin, 0, sm, 0, 0.0f};
+        const bt_status st = bt_forest_set_launch(f, &cfg);
+        if (st != BT_OK) {
+            cudaEventDestroy(e0);
+            cudaEventDestroy(e1);
+            return st;
+        }
+        walks[sm] = f->walk && nbatches <= kForestWalkList;
+    }
     bt_forest_tune b{};
     bool have = false;
     for (uint32_t w : warps)
         for (uint32_t p : pins)
             for (uint32_t lm = 0; lm <= 2 && e == cudaSuccess; ++lm)
                 for (uint32_t sm = 0; sm <= 2 && e == cudaSuccess; ++sm) {
+                    if (walks[sm] &&
+                        (w != kDefaultWarps || p != kDefaultPin || lm != 0 || (sm == 1 && walks[0])))
+                        continue;
                     const bt_forest_tune cfg{w, p, lm, sm, 0, 0.0f};
                     bt_status st = bt_forest_set_launch(f, &cfg);
                     if (st != BT_OK) {

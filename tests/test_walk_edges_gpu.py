@@ -203,3 +203,26 @@ def test_only_wholly_page_locked_queries_are_read_in_place(bt, locked):
         torch.cuda.synchronize()
         for at, _ in ranges[locked]:
             rt.cudaHostUnregister(q.ctypes.data + at * part)
+
+
+@pytest.mark.parametrize("staged", [False, True])
+def test_forest_autotune_times_the_walk_once(bt, staged):
+    """The settings that lead to the walk are one: the choice among them is
+    fixed and not the luckiest of many timings of the same launch."""
+    import torch
+    trees = _two_trees(bt)
+    if staged:  # the trees' own design no longer walks, reading through L1 does
+        bt.bt_tree_set_staging(trees[0][1].handle, bt.BT_STAGE_CP_ASYNC)
+    forest = bt.bt_forest_create([t[1].handle for t in trees])
+    nb, per = 200, 64
+    desc = np.zeros(nb, bt.BATCH_DESC_DTYPE)
+    desc["tree"], desc["count"], desc["offset"] = np.arange(nb) % 2, per, np.arange(nb) * per
+    q = _dev(W.make_queries(trees[1][0], nb * per, 0.8, seed=998, width_bits=64))
+    v, f = trees[0][1].alloc_outputs(nb * per)
+    wsb = bt.bt_forest_workspace_bytes(nb)
+    ws = torch.empty(wsb, dtype=torch.uint8, device="cuda")
+    best = bt.bt_forest_autotune(forest, _dev(desc.view(np.uint8)), nb, q, v, f, ws, wsb)
+    walk = (8, 16384, 0, 1 if staged else 0)
+    got = (best.warps_per_block, best.pin_budget, best.lane_queries, best.staging)
+    assert got == walk or best.staging == 2 or (staged and best.staging == 0)
+    bt.bt_forest_free(forest)
