@@ -131,21 +131,40 @@ typedef struct bt_info {
  * after the bytes all keys share).
  *
  * Behind the image (up to 8 MB of entries), or in an allocation of its own,
- * and not counted by bt_info, the device keeps a walk index: the keys and values once more in one-sector
+ * and not counted by bt_info (bt_tree_walk_bytes says how much it is), the
+ * device keeps a walk index: the keys and values once more in one-sector
  * entries (32-byte keys: 64 bytes each) under one-sector nodes, through which
  * batches are searched as given (see bt_search_opts.sort_bits).  It takes
  * about 18 bytes per 64-bit key and value (9 for 32-bit ones, 66 per 32-byte
- * key), more where keys crowd (up to 20, 10 and 72), and is left out when
- * that is above 32 MB and more than a quarter of the free device memory, or where the 8 bytes
- * after the bytes all 32-byte keys share are the same for hundreds of keys on
- * end; searches are then partitioned and descend the tree as bt_sort_bits
- * says.
+ * key), more where keys crowd (up to 20, 10 and 72).  It is left out on
+ * request (bt_build_ex), when it is above 32 MB and more than a quarter of the
+ * free device memory, or where the 8 bytes after the bytes all 32-byte keys
+ * share are the same for hundreds of keys on end; searches are then
+ * partitioned and descend the tree as bt_sort_bits says.
  *
  * Errors: BT_ERR_ARG, BT_ERR_FANOUT, BT_ERR_UNSORTED, BT_ERR_DUPLICATE,
  * BT_ERR_NOMEM, BT_ERR_CUDA.  *out is set only on BT_OK.
  */
 bt_status bt_build(const void *h_keys, const void *h_vals, uint64_t n, bt_width key_w,
                    bt_width val_w, uint32_t fanout, bt_stream stream, bt_tree **out);
+
+/* Options for bt_build_ex. */
+typedef struct bt_build_opts {
+    uint32_t walk_index; /* 1 (what bt_build does): build the walk index; 0: none, for
+                          * programs to which its memory (as much again as the tree) is
+                          * worth more than its speed (2^20 lookups over 2^24 64-bit
+                          * keys: 32 us with it, 91 without) */
+} bt_build_opts;
+
+/* bt_build with options (opts may be NULL = defaults).  Errors: as bt_build,
+ * BT_ERR_ARG also for an option out of range.  No counterpart in the paper. */
+bt_status bt_build_ex(const void *h_keys, const void *h_vals, uint64_t n, bt_width key_w,
+                      bt_width val_w, uint32_t fanout, const bt_build_opts *opts, bt_stream stream,
+                      bt_tree **out);
+
+/* Bytes of device memory the tree holds for its walk index besides
+ * bt_info.device_bytes; 0 for a NULL tree.  No counterpart in the paper. */
+uint64_t bt_tree_walk_bytes(const bt_tree *tree);
 
 /* Release a tree and its device memory (NULL is a no-op).  The caller must
  * make sure no search using it is still running.  No counterpart in the

@@ -30,20 +30,21 @@ STATUS = {0: "BT_OK", 1: "BT_ERR_ARG", 2: "BT_ERR_UNSORTED", 3: "BT_ERR_DUPLICAT
           8: "BT_ERR_WORKSPACE"}
 
 # Every symbol include/btree_gb300.h declares.
-EXPORTED = ("bt_build", "bt_free", "bt_tree_info", "bt_tree_copy_image", "bt_search_workspace_bytes",
-            "bt_search_batch", "bt_search_batch_ex", "bt_sort_batch", "bt_descend_sorted", "bt_sort_launches", "bt_sort_bits",
-            "bt_search_host_workspace_bytes",
+EXPORTED = ("bt_build", "bt_build_ex", "bt_tree_walk_bytes", "bt_free", "bt_tree_info", "bt_tree_copy_image",
+            "bt_search_workspace_bytes", "bt_search_batch", "bt_search_batch_ex", "bt_sort_batch",
+            "bt_descend_sorted", "bt_sort_launches", "bt_sort_bits", "bt_search_host_workspace_bytes",
             "bt_search_batch_host", "bt_search_batch_noalloc", "bt_status_str", "bt_last_error_detail",
             "bt_model_train", "bt_model_free", "bt_model_get_info", "bt_model_copy_params", "bt_mlp_grad",
             "bt_learned_descend_sorted", "bt_learned_search_batch", "bt_model_copy_err_bounds",
             "bt_forest_create", "bt_forest_create_learned", "bt_forest_free", "bt_forest_set_launch",
-            "bt_forest_get_launch", "bt_forest_autotune", "bt_forest_workspace_bytes", "bt_forest_search", "bt_forest_bad_batches", "bt_tree_set_launch", "bt_tree_set_staging",
-            "bt_tree_set_lane_queries", "bt_tree_set_descent", "bt_tree_set_l2_window", "bt_tree_set_corun", "bt_debug_set_wait_polls",
+            "bt_forest_get_launch", "bt_forest_autotune", "bt_forest_workspace_bytes", "bt_forest_search",
+            "bt_forest_bad_batches", "bt_tree_set_launch", "bt_tree_set_staging", "bt_tree_set_lane_queries",
+            "bt_tree_set_descent", "bt_tree_set_l2_window", "bt_tree_set_corun", "bt_debug_set_wait_polls",
             "bt_check_timeouts", "bt_autotune", "bt_paper_node_bytes", "bt_paper_layout_build",
-            "bt_paper_search_batch", "bt_paper_descend_sorted",
-            "bt_server_create", "bt_server_submit", "bt_server_poll", "bt_server_drain", "bt_server_get_stats",
-            "bt_server_destroy", "bt_server_run_trace", "bt_range_build", "bt_range_free", "bt_range_info",
-            "bt_range_part", "bt_range_workspace_bytes", "bt_range_search")
+            "bt_paper_search_batch", "bt_paper_descend_sorted", "bt_server_create", "bt_server_submit",
+            "bt_server_poll", "bt_server_drain", "bt_server_get_stats", "bt_server_destroy",
+            "bt_server_run_trace", "bt_range_build", "bt_range_free", "bt_range_info", "bt_range_part",
+            "bt_range_workspace_bytes", "bt_range_search")
 
 
 class bt_info(ctypes.Structure):
@@ -62,9 +63,18 @@ class bt_search_opts(ctypes.Structure):
     _fields_ = [("sort_bits", ctypes.c_int32), ("d_fetch_counts", ctypes.c_void_p), ("phase_event", ctypes.c_void_p)]
 
 
+class bt_build_opts(ctypes.Structure):
+    _fields_ = [("walk_index", ctypes.c_uint32)]
+
+
 _vp, _u64, _i = ctypes.c_void_p, ctypes.c_uint64, ctypes.c_int
 _lib.bt_build.restype = _i
 _lib.bt_build.argtypes = [_vp, _vp, _u64, _i, _i, ctypes.c_uint32, _vp, ctypes.POINTER(_vp)]
+_lib.bt_build_ex.restype = _i
+_lib.bt_build_ex.argtypes = [_vp, _vp, _u64, _i, _i, ctypes.c_uint32, ctypes.POINTER(bt_build_opts), _vp,
+                             ctypes.POINTER(_vp)]
+_lib.bt_tree_walk_bytes.restype = _u64
+_lib.bt_tree_walk_bytes.argtypes = [_vp]
 _lib.bt_free.restype = None
 _lib.bt_free.argtypes = [_vp]
 _lib.bt_tree_info.restype = _i
@@ -164,9 +174,10 @@ def bt_status_str(status: int) -> str:
     return _lib.bt_status_str(status).decode()
 
 
-def bt_build(h_keys: np.ndarray, h_vals: np.ndarray, fanout: int, stream=None) -> int:
+def bt_build(h_keys: np.ndarray, h_vals: np.ndarray, fanout: int, stream=None, walk_index: bool = True) -> int:
     """Bulk-load a tree from sorted host keys/values; returns the opaque handle.
-    Keys: a 1-D uint32/uint64 array, or an (n, 32) uint8 array of 32-byte keys."""
+    Keys: a 1-D uint32/uint64 array, or an (n, 32) uint8 array of 32-byte keys.
+    walk_index=False: without the walk index and its memory (bt_build_ex)."""
     k = np.ascontiguousarray(h_keys)
     v = np.ascontiguousarray(h_vals)
     if k.ndim == 2 and k.dtype == np.uint8 and k.shape[1] == 32:
@@ -178,10 +189,15 @@ def bt_build(h_keys: np.ndarray, h_vals: np.ndarray, fanout: int, stream=None) -
     if v.ndim != 1 or v.size != n:
         raise ValueError("values must be a 1-D array with one value per key")
     out = _vp()
-    st = _lib.bt_build(k.ctypes.data if n else None, v.ctypes.data if n else None,
-                       n, kw, _width(v.dtype), fanout, _stream_handle(stream), ctypes.byref(out))
+    opts = bt_build_opts(1 if walk_index else 0)
+    st = _lib.bt_build_ex(k.ctypes.data if n else None, v.ctypes.data if n else None, n, kw, _width(v.dtype),
+                          fanout, ctypes.byref(opts), _stream_handle(stream), ctypes.byref(out))
     _check("bt_build", st)
     return out.value
+
+
+def bt_tree_walk_bytes(tree: int) -> int:
+    return int(_lib.bt_tree_walk_bytes(tree))
 
 
 def bt_free(tree: int) -> None:
@@ -687,9 +703,9 @@ class BTree:
     """A tree on the current CUDA device with convenience search methods."""
 
     def __init__(self, keys: np.ndarray | None, vals: np.ndarray | None, fanout: int = 0, stream=None,
-                 handle: int | None = None):
+                 handle: int | None = None, walk_index: bool = True):
         """Build from sorted keys/values, or take ownership of a built tree's handle."""
-        self.handle = handle if handle is not None else bt_build(keys, vals, fanout, stream)
+        self.handle = handle if handle is not None else bt_build(keys, vals, fanout, stream, walk_index)
         i = bt_tree_info(self.handle)
         self.height = int(i.height)
         self.fanout = int(i.fanout)

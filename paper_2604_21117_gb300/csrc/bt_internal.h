@@ -85,7 +85,7 @@ constexpr int kWalkLevels = 12;
 struct WalkDev {
     const unsigned char *top;      // separators of the segments, bin table, octave table
     const unsigned char *nodes;    // 32-byte nodes, level 0 (one node per segment) first
-    const unsigned char *entries;  // 64-byte entries
+    const unsigned char *entries;  // 32-byte entries (32-byte keys: 64)
     uint64_t off[kWalkLevels];     // byte offset of each level in nodes
     uint64_t n;                    // keys
     uint64_t wmin, wmax;           // smallest and largest key (32-byte keys: word)
@@ -129,6 +129,7 @@ struct bt_tree {
     btgb::WalkDev walk;  // valid while d_walk is set
     void *d_walk;        // the walk index (null: not built)
     bool walk_own;       // it is an allocation of its own, not part of the image's
+    uint64_t walk_bytes; // device memory held for it, there or behind the image
 };
 
 struct bt_model {

@@ -274,7 +274,16 @@ extern "C" const char *bt_status_str(bt_status s)
 extern "C" bt_status bt_build(const void *h_keys, const void *h_vals, uint64_t n, bt_width key_w,
                               bt_width val_w, uint32_t fanout, bt_stream stream, bt_tree **out)
 {
+    return bt_build_ex(h_keys, h_vals, n, key_w, val_w, fanout, nullptr, stream, out);
+}
+
+extern "C" bt_status bt_build_ex(const void *h_keys, const void *h_vals, uint64_t n, bt_width key_w,
+                                 bt_width val_w, uint32_t fanout, const bt_build_opts *opts, bt_stream stream,
+                                 bt_tree **out)
+{
     if (!out) return BT_ERR_ARG;
+    if (opts && opts->walk_index > 1) return BT_ERR_ARG;
+    const bool walk = !opts || opts->walk_index == 1;
     if ((key_w != BT_U32 && key_w != BT_U64 && key_w != BT_B32) || (val_w != BT_U32 && val_w != BT_U64))
         return BT_ERR_ARG;
     if (fanout != 8 && fanout != 16 && fanout != 32 && fanout != 64) return BT_ERR_FANOUT;
@@ -487,7 +496,7 @@ extern "C" bt_status bt_build(const void *h_keys, const void *h_vals, uint64_t n
     }
 
     // a small tree's walk index lies behind the image
-    uint64_t room = walk_room(n, kb, vb);
+    uint64_t room = walk ? walk_room(n, kb, vb) : 0;
     cudaError_t e = cudaMalloc(&t->d_image, off + room);
     if (e == cudaErrorMemoryAllocation && room) {
         cudaGetLastError();
@@ -518,7 +527,8 @@ extern "C" bt_status bt_build(const void *h_keys, const void *h_vals, uint64_t n
     d.split_off = kb == 32 ? static_cast<unsigned char *>(t->d_image) + split_off_offset : nullptr;
     d.split_R = reinterpret_cast<const uint16_t *>(static_cast<unsigned char *>(t->d_image) + split_R_offset);
     t->info.d_image = t->d_image;
-    e = walk_build(t, h_keys, room ? static_cast<unsigned char *>(t->d_image) + off : nullptr, room, s);
+    t->walk_bytes = room;
+    if (walk) e = walk_build(t, h_keys, room ? static_cast<unsigned char *>(t->d_image) + off : nullptr, room, s);
     if (e != cudaSuccess) {
         set_error_detail("walk index", e);
         bt_free(t);
@@ -527,6 +537,8 @@ extern "C" bt_status bt_build(const void *h_keys, const void *h_vals, uint64_t n
     *out = t;
     return BT_OK;
 }
+
+extern "C" uint64_t bt_tree_walk_bytes(const bt_tree *t) { return t ? t->walk_bytes : 0; }
 
 extern "C" void bt_free(bt_tree *t)
 {

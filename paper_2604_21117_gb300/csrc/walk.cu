@@ -372,6 +372,7 @@ cudaError_t walk_build(bt_tree *t, const void *h_keys, unsigned char *d_room, ui
         e = cudaMalloc(&t->d_walk, bytes);
     else
         t->d_walk = d_room;
+    if (t->walk_own && e == cudaSuccess) t->walk_bytes += bytes;
     if (e == cudaErrorMemoryAllocation) {
         cudaGetLastError();  // searched by the descent, as without this index
         t->d_walk = nullptr;
