@@ -226,3 +226,127 @@ def test_forest_autotune_times_the_walk_once(bt, staged):
     got = (best.warps_per_block, best.pin_budget, best.lane_queries, best.staging)
     assert got == walk or best.staging == 2 or (staged and best.staging == 0)
     bt.bt_forest_free(forest)
+
+
+# Keys per entry: 32 / (key + value bytes).  Up to 2^12 entries the top alone,
+# then one coded level of 17 children up to 2^12 segments, then two, then from
+# 15360 segments (25600 for 32-bit keys) a level of full words above those.
+def _per_entry(kw, vw):
+    return 32 // ((kw + vw) // 8)
+
+
+def _expect(keys, vw, q):
+    pos = np.searchsorted(keys, q)
+    hit = keys[np.minimum(pos, keys.size - 1)] == q
+    return np.where(hit, pos.astype(np.uint64), np.uint64(2**vw - 1)), hit
+
+
+def _edge_queries(keys, kw, vw, seed):
+    """Keys at the ends of entries, nodes and segments and the values beside
+    them, random keys, random values."""
+    G, n, g = _per_entry(kw, vw), keys.size, W.rng(seed)
+    ranks = [g.integers(0, n, size=40_000)]
+    for span in (1, 17, 289, 289 * 5, 289 * 9):
+        ends = np.arange(1, n // (span * G) + 1) * (span * G)
+        ends = ends if ends.size < 20_000 else np.concatenate([ends[:5000], ends[-5000:], g.choice(ends, 10_000)])
+        ranks += [ends - 1, np.minimum(ends, n - 1), np.minimum(ends + 1, n - 1)]
+    k = keys[np.concatenate(ranks + [np.array([0, n - 1])])]
+    return np.concatenate([k, k + keys.dtype.type(1), k - keys.dtype.type(1),
+                           g.integers(0, 2**kw, size=2000, dtype=np.uint64).astype(keys.dtype)])
+
+
+@pytest.mark.parametrize("kw,vw", [(64, 64), (64, 32), (32, 64), (32, 32)])
+@pytest.mark.parametrize("entries,more", [(1, 0), (1, 1), (4096, 0), (4096, 1), (17 * 4096, 0), (17 * 4096, 1)])
+def test_where_the_index_changes_shape(bt, kw, vw, entries, more):
+    n = _per_entry(kw, vw) * entries + more
+    keys = W.uniform_keys(n, kw, seed=1020 + n)
+    tree = bt.BTree(keys, W.rank_values(n, vw), 16)
+    q = _edge_queries(keys, kw, vw, 1021)
+    want, hit = _expect(keys, vw, q)
+    for nq in (1, 33, q.size):
+        v, f = tree.search(_dev(q[-nq:]))
+        assert np.array_equal(v.cpu().numpy().astype(np.uint64), want[-nq:])
+        assert np.array_equal(f.cpu().numpy().astype(bool), hit[-nq:])
+
+
+@pytest.mark.parametrize("kw,vw,segs", [(64, 64, 15360), (32, 64, 25600), (32, 32, 25600)])
+@pytest.mark.parametrize("more", [0, 3])
+def test_full_words_above_coded_levels(bt, kw, vw, segs, more):
+    """The largest top over two coded levels, and the smallest trees with a
+    level of full words between them."""
+    n = _per_entry(kw, vw) * 289 * segs + more
+    keys = W.uniform_keys(n, kw, seed=1022)
+    tree = bt.BTree(keys, W.rank_values(n, vw), 64)
+    q = _edge_queries(keys, kw, vw, 1023)
+    want, hit = _expect(keys, vw, q)
+    v, f = tree.search(_dev(q))
+    assert np.array_equal(v.cpu().numpy().astype(np.uint64), want)
+    assert np.array_equal(f.cpu().numpy().astype(bool), hit)
+    tree.close()
+
+
+@pytest.mark.parametrize("ties", ["few", "many"])
+def test_full_words_of_byte_keys_that_tie(bt, ties):
+    """Words that tie across the ends of nodes and segments, in so few keys
+    that the lower levels stay coded and in so many that none is."""
+    n = 289 * 15360 + 3
+    words = W.uniform_keys(n, 64, seed=1024).astype(np.uint64)
+    second = np.arange(1445, n, 1445) if ties == "few" else np.arange(3, n, 3)
+    words[second] = words[second - 1]
+    keys = np.zeros((n, 32), np.uint8)
+    keys[:, :8] = words.astype(">u8").view(np.uint8).reshape(n, 8)
+    keys[:, 31] = 1
+    keys[second, 31] = 3
+    tree = bt.BTree(keys, W.rank_values(n, 64), 64)
+    assert bt.bt_tree_walk_bytes(tree.handle) > 0
+    g = W.rng(1025)
+    at = np.concatenate([second[:30_000] - 1, second[:30_000], second[-30_000:], g.integers(0, n, size=60_000),
+                         np.array([0, n - 1])])
+    q = np.concatenate([keys[at]] * 3)
+    q[at.size: 2 * at.size, 31] += 1   # between the two of a pair, or above it: stored nowhere
+    q[2 * at.size:, 31] = 0            # below both
+    v, f = tree.search(_dev(q))
+    v, f = v.cpu().numpy(), f.cpu().numpy()
+    assert np.array_equal(v[: at.size], at.astype(np.uint64)) and f[: at.size].all()
+    assert (v[at.size:] == np.uint64(2**64 - 1)).all() and not f[at.size:].any()
+    tree.close()
+
+
+@pytest.mark.parametrize("ntrees", [128, 129])
+def test_as_many_trees_as_the_walks_table_holds_and_one_more(bt, ntrees):
+    import torch
+    keysets = [W.uniform_keys(20 + 37 * i, 64, seed=1026 + i) for i in range(ntrees)]
+    trees = [bt.BTree(k, W.rank_values(k.size, 64), 16) for k in keysets]
+    forest = bt.bt_forest_create([t.handle for t in trees])
+    per = 45
+    desc = np.zeros(ntrees, bt.BATCH_DESC_DTYPE)
+    desc["tree"], desc["count"], desc["offset"] = np.arange(ntrees), per, np.arange(ntrees) * per
+    q = np.concatenate([W.make_queries(k, per, 0.7, seed=1027, width_bits=64) for k in keysets])
+    v, f = trees[0].alloc_outputs(q.size)
+    wsb = bt.bt_forest_workspace_bytes(ntrees)
+    bt.bt_forest_search(forest, _dev(desc.view(np.uint8)), ntrees, _dev(q), v, f,
+                        torch.empty(wsb, dtype=torch.uint8, device="cuda"), wsb)
+    want = [_expect(k, 64, q[i * per:(i + 1) * per]) for i, k in enumerate(keysets)]
+    assert np.array_equal(v.cpu().numpy(), np.concatenate([w[0] for w in want]))
+    assert np.array_equal(f.cpu().numpy().astype(bool), np.concatenate([w[1] for w in want]))
+    bt.bt_forest_free(forest)
+
+
+@pytest.mark.parametrize("kind", ["pl", "pl_many", "mlp"])
+@pytest.mark.parametrize("kw,entries", [(64, 4096), (64, 17 * 4096), (32, 4096), (32, 17 * 4096)])
+def test_learned_search_where_the_index_changes_shape(bt, kind, kw, entries):
+    n = _per_entry(kw, 64) * entries + 1
+    keys = W.lognormal_mixture_keys(n, seed=1028) if kw == 64 else W.uniform_keys(n, kw, seed=1028)
+    tree = bt.BTree(keys, W.rank_values(n, 64), 32)
+    if kind == "mlp":
+        m = bt.bt_model_train(tree.handle, bt.BT_MODEL_MLP, h_init=W.mlp_init_params(1029), steps=20, batch=1024,
+                              lr=2e-3, seed=1030)
+    else:
+        m = bt.bt_model_train(tree.handle, bt.BT_MODEL_PL, segments={"pl": 64, "pl_many": 2000}[kind])
+    q = _edge_queries(keys, kw, 64, 1031)
+    want, hit = _expect(keys, 64, q)
+    v, f = tree.alloc_outputs(q.size)
+    ws, nb = tree.alloc_workspace(q.size)
+    bt.bt_learned_search_batch(tree.handle, m, _dev(q), q.size, v, f, ws, nb)
+    assert np.array_equal(v.cpu().numpy(), want) and np.array_equal(f.cpu().numpy().astype(bool), hit)
+    bt.bt_model_free(m)
