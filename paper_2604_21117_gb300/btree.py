@@ -129,20 +129,23 @@ def _check(call: str, st: int):
 _raw_stream = _current_device = None
 
 
-def _stream_handle(stream) -> int | None:
+def _first_stream_handle() -> int:
+    """The current stream's handle, CUDA brought up, and the two lookups set."""
     global _raw_stream, _current_device
+    import torch
+    handle = torch.cuda.current_stream().cuda_stream
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    device = getattr(torch._C, "_cuda_getDevice", None)
+    if raw is None or device is None:
+        raw, device = (lambda _: torch.cuda.current_stream().cuda_stream), (lambda: 0)
+    _raw_stream = raw
+    _current_device = device
+    return handle
+
+
+def _stream_handle(stream) -> int | None:
     if stream is None:
-        if _current_device is None:
-            import torch
-            handle = torch.cuda.current_stream().cuda_stream
-            raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
-            device = getattr(torch._C, "_cuda_getDevice", None)
-            if raw is None or device is None:
-                raw, device = (lambda _: torch.cuda.current_stream().cuda_stream), (lambda: 0)
-            _raw_stream = raw
-            _current_device = device
-            return handle
-        return _raw_stream(_current_device())
+        return _first_stream_handle() if _current_device is None else _raw_stream(_current_device())
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
