@@ -192,9 +192,10 @@ def bt_build(h_keys: np.ndarray, h_vals: np.ndarray, fanout: int, stream=None, w
     if v.ndim != 1 or v.size != n:
         raise ValueError("values must be a 1-D array with one value per key")
     out = _vp()
-    opts = bt_build_opts(1 if walk_index else 0)
+    # (bt_build_ex with no options is bt_build)
+    opts = None if walk_index else ctypes.byref(bt_build_opts(0))
     st = _lib.bt_build_ex(k.ctypes.data if n else None, v.ctypes.data if n else None, n, kw, _width(v.dtype),
-                          fanout, ctypes.byref(opts), _stream_handle(stream), ctypes.byref(out))
+                          fanout, opts, _stream_handle(stream), ctypes.byref(out))
     _check("bt_build", st)
     return out.value
 

@@ -271,19 +271,10 @@ extern "C" const char *bt_status_str(bt_status s)
     return "unknown status";
 }
 
-extern "C" bt_status bt_build(const void *h_keys, const void *h_vals, uint64_t n, bt_width key_w,
-                              bt_width val_w, uint32_t fanout, bt_stream stream, bt_tree **out)
-{
-    return bt_build_ex(h_keys, h_vals, n, key_w, val_w, fanout, nullptr, stream, out);
-}
-
-extern "C" bt_status bt_build_ex(const void *h_keys, const void *h_vals, uint64_t n, bt_width key_w,
-                                 bt_width val_w, uint32_t fanout, const bt_build_opts *opts, bt_stream stream,
-                                 bt_tree **out)
+static bt_status build_tree(const void *h_keys, const void *h_vals, uint64_t n, bt_width key_w, bt_width val_w,
+                            uint32_t fanout, bool walk, bt_stream stream, bt_tree **out)
 {
     if (!out) return BT_ERR_ARG;
-    if (opts && opts->walk_index > 1) return BT_ERR_ARG;
-    const bool walk = !opts || opts->walk_index == 1;
     if ((key_w != BT_U32 && key_w != BT_U64 && key_w != BT_B32) || (val_w != BT_U32 && val_w != BT_U64))
         return BT_ERR_ARG;
     if (fanout != 8 && fanout != 16 && fanout != 32 && fanout != 64) return BT_ERR_FANOUT;
@@ -536,6 +527,20 @@ extern "C" bt_status bt_build_ex(const void *h_keys, const void *h_vals, uint64_
     }
     *out = t;
     return BT_OK;
+}
+
+extern "C" bt_status bt_build(const void *h_keys, const void *h_vals, uint64_t n, bt_width key_w,
+                              bt_width val_w, uint32_t fanout, bt_stream stream, bt_tree **out)
+{
+    return build_tree(h_keys, h_vals, n, key_w, val_w, fanout, true, stream, out);
+}
+
+extern "C" bt_status bt_build_ex(const void *h_keys, const void *h_vals, uint64_t n, bt_width key_w,
+                                 bt_width val_w, uint32_t fanout, const bt_build_opts *opts, bt_stream stream,
+                                 bt_tree **out)
+{
+    if (opts && opts->walk_index > 1) return BT_ERR_ARG;
+    return build_tree(h_keys, h_vals, n, key_w, val_w, fanout, !opts || opts->walk_index == 1, stream, out);
 }
 
 extern "C" uint64_t bt_tree_walk_bytes(const bt_tree *t) { return t ? t->walk_bytes : 0; }
