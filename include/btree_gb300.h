@@ -195,13 +195,13 @@ typedef struct bt_search_opts {
      * (larger values mean 21).  A batch that is not forced goes through the
      * tree's walk index as given, the faster way at every size, unless the
      * tree has none, d_fetch_counts is set, its results lie over its queries
-     * (see bt_search_batch), or another descent than the
-     * pipelined one with the binary-search rank has been chosen for it
-     * (bt_tree_set_staging, bt_tree_set_lane_queries, bt_tree_set_descent);
-     * then -1 partitions on bt_sort_bits bits (none below 786432 queries --
-     * 393216 for 32-byte keys -- and none for a tree whose device image is at
-     * most a quarter of the L2: the partition pays for itself only when the
-     * batch is large and leaf blocks do not stay in the L2 between batches). */
+     * (see bt_search_batch), or another descent than the pipelined one with
+     * the binary-search rank has been chosen for it (bt_tree_set_staging,
+     * bt_tree_set_lane_queries, bt_tree_set_descent); then -1 partitions on
+     * bt_sort_bits bits (none below 786432 queries -- 393216 for 32-byte
+     * keys -- and none for a tree whose device image is at most a quarter
+     * of the L2: the partition pays for itself only when the batch is large
+     * and leaf blocks do not stay in the L2 between batches). */
     int32_t sort_bits;
     /* If non-NULL: device array of `height` counters to which the search
      * adds, per level, how many node key blocks it fetched -- the quantity
@@ -297,7 +297,8 @@ int32_t bt_sort_launches(const bt_tree *tree, uint64_t nq, int32_t sort_bits);
 
 /* Bits of the bucket number f that bt_sort_batch, and a bt_search_batch that
  * does not go through the walk index, order a batch of nq queries on, for
- * this sort_bits (-1 = the library's choice); 0 = no partition.  -1 on a NULL tree.  No counterpart in the paper. */
+ * this sort_bits (-1 = the library's choice); 0 = no partition.  -1 on a NULL
+ * tree.  No counterpart in the paper. */
 int32_t bt_sort_bits(const bt_tree *tree, uint64_t nq, int32_t sort_bits);
 
 /*
@@ -405,10 +406,13 @@ typedef struct bt_forest bt_forest;
  * ones are staged per warp (the synchronous designs and inner-staged
  * pipelined design) or read lane by lane through L1 (the pipelined design).
  * Warps per block default to the setting of the tree with the most keys,
- * the pin budget to 32 KB.  A forest none of whose trees is staged per warp,
- * and all of whose trees have a walk index (see bt_build), searches them
- * through it instead, in chunks of 32 queries and blocks of its own shape:
- * those settings then have no effect.  The trees must outlive the forest.
+ * the pin budget to 32 KB.  A forest of at most 128 trees, none of which is
+ * staged per warp or has a model and all of which have a walk index (see
+ * bt_build), searches them through it instead, in chunks of 32 queries and
+ * blocks of its own shape: those settings then have no effect (lists of more
+ * than 65536 batches in device memory still descend, under them).  One tree
+ * that is otherwise makes the whole forest descend, at about a third of the
+ * speed.  The trees must outlive the forest.
  * Errors: BT_ERR_ARG, BT_ERR_NOMEM, BT_ERR_CUDA. */
 bt_status bt_forest_create(const bt_tree *const *trees, uint32_t count, bt_forest **out);
 
@@ -507,7 +511,9 @@ typedef struct bt_tune {
  * top levels each block keeps in shared memory (0..49152).  The pipelined
  * descent gives a batch with fewer 32-query chunks per SM than
  * warps_per_block smaller blocks (that many warps, at least 2), so that a
- * small batch spreads over more SMs.  BT_ERR_ARG on unsupported values. */
+ * small batch spreads over more SMs.  A batch that goes through the walk index
+ * (see bt_search_opts.sort_bits) runs in a launch of its own shape, which
+ * neither setting touches.  BT_ERR_ARG on unsupported values. */
 bt_status bt_tree_set_launch(bt_tree *tree, uint32_t warps_per_block, uint32_t pin_bytes);
 
 /* How the descent stages node blocks into shared memory (Sec. IV-A: every
@@ -536,6 +542,8 @@ bt_status bt_tree_set_staging(bt_tree *tree, uint32_t mode);
  *                 memory once with 16-byte cp.async, then searched there;
  *                 2 (default): 1 for partitioned batches (a warp meets one or
  *                 two nodes per level), 0 for unsorted ones (up to 32).
+ *                 Of no effect on batches that go through the walk index
+ *                 (see bt_search_opts.sort_bits).
  *   rank_ballot   0 (default): each query finds its leaf rank by binary
  *                 search in the staged block; 1: the rank is the population
  *                 count of a warp ballot, lane j comparing slot j (and j+32)
@@ -547,8 +555,9 @@ bt_status bt_tree_set_descent(bt_tree *tree, uint32_t inner_staged, uint32_t ran
 /* An L2 access-policy window for the tree's searches: the inner levels below
  * the shared-memory-pinned ones (at most max_bytes, and at most the device's
  * window size) are marked persisting in L2 on every descent launch, so that
- * the stream of leaf blocks does not evict them between batches.  Sets this
- * process's persisting-L2 set-aside (cudaLimitPersistingL2CacheSize) to at
+ * the stream of leaf blocks does not evict them between batches.  Batches that
+ * go through the walk index (see bt_search_opts.sort_bits) read none of those
+ * levels and get no window.  Sets this process's persisting-L2 set-aside (cudaLimitPersistingL2CacheSize) to at
  * least the window's size if it is smaller; the set-aside belongs to this
  * process's CUDA context and ends with it.  0 removes the window.  No
  * counterpart in the paper (its top levels stay on chip, Sec. IV-A).
@@ -593,8 +602,9 @@ bt_status bt_tree_set_lane_queries(bt_tree *tree, uint32_t per_lane);
 
 /* BT_ERR_TIMEOUT if a bounded device wait of a search gave up since the
  * last call (the results of such a search are invalid, those of a work list
- * excepted: see bt_debug_set_wait_polls), else BT_OK; clears the counters.  Synchronous (reads device counters).  No counterpart in the
- * paper (its kernel has no waits that can fail). */
+ * excepted: see bt_debug_set_wait_polls), else BT_OK; clears the counters.
+ * Synchronous (reads device counters).  No counterpart in the paper (its
+ * kernel has no waits that can fail). */
 bt_status bt_check_timeouts(void);
 
 /*
@@ -605,9 +615,9 @@ bt_status bt_check_timeouts(void);
  * through L1 or staged; synchronous with cp.async or bulk-copy staging; two
  * queries per lane); keep the fastest.  The pipelined settings search the
  * sample through the walk index, on which none of them bears: they are timed
- * once per fanout, at 8 warps and 16384 pinned bytes.  *out receives the tree built with
- * the best fanout and launch parameters applied, *best the choice and its
- * time.  A sample with fewer 32-query chunks per SM than a warps-per-block
+ * once per fanout, at 8 warps and 16384 pinned bytes.  *out receives the tree
+ * built with the best fanout and launch parameters applied, *best the choice
+ * and its time.  A sample with fewer 32-query chunks per SM than a warps-per-block
  * setting runs the pipelined descent in smaller blocks whatever that setting
  * is (see bt_tree_set_launch), so such settings are not tried for it and the
  * pipelined designs keep 8 warps per block: tune on a batch of the size the

@@ -65,9 +65,10 @@ constexpr uint32_t kForestSmemList = 64;  // work lists up to this long are read
 constexpr uint32_t kForestPinMax = 98304;
 constexpr int kForestSmemMax = 200 * 1024;
 // Tops of a forest's trees in shared memory.  10,000 batches over trees of
-// 10^3, 10^5, 10^6 and 2 * 10^7 uint64 keys, with tops searched by bisection
-// (146 KB): 58.9 us with all of them there, 71.7 with 96 KB (the largest
-// tree's top through L1), 68.9 with none.
+// 10^3, 10^5, 10^6 and 2 * 10^7 uint64 keys: 58.9 us with all of them there,
+// 71.7 with 96 KB (the largest tree's top through L1), 68.9 with none.  That
+// was measured on this one list, and with an earlier form of the tops (searched
+// by bisection, 146 KB; the same trees' are 112 KB now).
 constexpr uint32_t kWalkTopBudget = 128 * 1024;
 
 __host__ __device__ inline uint32_t forest_desc_chunks(const bt_batch_desc &bd, uint32_t ntrees, uint64_t nq,
@@ -565,7 +566,8 @@ static std::vector<ForestWalk> walk_table(bt_forest *f)
         // single chunk's latency grows less than that; in between, so that
         // both the blocks and the warps in them end together (10,000 batches:
         // 43.8 us so, 47.2 with the list times as costs, 46.7 with 28 + 6 per
-        // level).
+        // level).  Measured on this list alone; 32-bit trees get the same
+        // weights.  They only shift load: any others give the same results.
         const uint64_t entry_bytes = tab[i].w.n / walk_group(f->key_bytes, f->val_bytes) * 32;
         tab[i].cost = 20u + 8u * static_cast<uint32_t>(tab[i].w.levels) + (entry_bytes > (64u << 20) ? 6u : 0u);
     }

@@ -58,8 +58,8 @@ __device__ __forceinline__ uint64_t warp_incl_scan(uint64_t x, uint32_t lane)
     return x;
 }
 
-// Shared memory: the tops that have a place (top_total bytes), the table, then (lists without chunk offsets) the
-// positions of the list's rows.
+// Shared memory: the tops that have a place (top_total bytes), the table, then
+// (lists without chunk offsets) the positions of the list's rows.
 template <typename K, typename V>
 __global__ void __launch_bounds__(kWalkForestThreads)
     k_forest_walk(const ForestWalk *__restrict__ gtab, uint32_t ntrees, uint32_t top_total,
@@ -95,7 +95,8 @@ __global__ void __launch_bounds__(kWalkForestThreads)
         for (uint32_t r0 = warp; r0 < nrows; r0 += nw * U) {
             Entry e[U];
 #pragma unroll
-            for (int u = 0; u < U; ++u) e[u] = list_entry(batches, (r0 + u * nw) * 32 + lane, nb, tab, ntrees, nq, false);
+            for (int u = 0; u < U; ++u)
+                e[u] = list_entry(batches, (r0 + u * nw) * 32 + lane, nb, tab, ntrees, nq, false);
 #pragma unroll
             for (int u = 0; u < U; ++u) {
                 // at most 2^27 chunks of a cost below 2^12: two sums below 2^32
@@ -297,11 +298,9 @@ cudaError_t forest_walk_run(const ForestWalk *tab, uint32_t ntrees, uint32_t top
                             const bt_batch_desc *b, uint32_t nb, const uint32_t *cs, uint32_t host_chunks,
                             const void *q, uint64_t nq, void *ov, uint8_t *of, cudaStream_t s, ForestDone done)
 {
-    if (kb == 8)
-        return vb == 8 ? walk_forest_launch<uint64_t, uint64_t>(tab, ntrees, top_total, b, nb, cs, host_chunks, q, nq, ov, of, s, done)
-                       : walk_forest_launch<uint64_t, uint32_t>(tab, ntrees, top_total, b, nb, cs, host_chunks, q, nq, ov, of, s, done);
-    return vb == 8 ? walk_forest_launch<uint32_t, uint64_t>(tab, ntrees, top_total, b, nb, cs, host_chunks, q, nq, ov, of, s, done)
-                   : walk_forest_launch<uint32_t, uint32_t>(tab, ntrees, top_total, b, nb, cs, host_chunks, q, nq, ov, of, s, done);
+    auto launch = kb == 8 ? (vb == 8 ? walk_forest_launch<uint64_t, uint64_t> : walk_forest_launch<uint64_t, uint32_t>)
+                          : (vb == 8 ? walk_forest_launch<uint32_t, uint64_t> : walk_forest_launch<uint32_t, uint32_t>);
+    return launch(tab, ntrees, top_total, b, nb, cs, host_chunks, q, nq, ov, of, s, done);
 }
 
 cudaError_t take_wait_counters_forest(unsigned *timeouts, unsigned *pending)

@@ -270,8 +270,9 @@ static std::vector<unsigned char> build_top(WalkDev &w, const std::vector<uint64
 // Up to 8 MB of entries share the image's allocation: one cudaMalloc and one
 // cudaFree less (247,326 uint64 keys: bt_build 0.95 -> 0.78 ms, 0.74 without
 // an index, bt_free 95 -> 67 us; 50,000 32-byte keys, whose check for ties
-// then needs no allocation either: 0.79 -> 0.63 and 0.55 ms).  The most the index can take: the largest top, full-word
-// nodes (a fifth of the entries, and again), the entries.
+// then needs no allocation either: 0.79 -> 0.63 and 0.55 ms).  The most the
+// index can take: the largest top, full-word nodes (a fifth of the entries,
+// and again), the entries.
 uint64_t walk_room(uint64_t n, int key_bytes, int val_bytes)
 {
     const uint64_t G = walk_group(key_bytes, val_bytes), E = (n + G - 1) / G;
@@ -547,14 +548,16 @@ __global__ void __launch_bounds__(walk_threads<MODEL>())
             uint32_t lo, hi;
             // (two calls, so that each reads the parameters by their own address space)
             if (MODEL == kModelMLP || walk_model_bytes(m.md))
-                model_window<MODEL>(m.md, walk_model<MODEL>(m.md, smem + w.top_bytes), static_cast<uint64_t>(key), lo, hi);
+                model_window<MODEL>(m.md, walk_model<MODEL>(m.md, smem + w.top_bytes), static_cast<uint64_t>(key), lo,
+                                    hi);
             else
                 model_window<MODEL>(m.md, ModelView{m.md.b, m.md.inv_w, m.md.slope, m.md.icpt, m.md.mlp, nullptr},
                                     static_cast<uint64_t>(key), lo, hi);
             // first key of leaf lo, last key of leaf hi, as entries, as segments
             const uint64_t r0 = lo * m.leaf_base + (lo < m.leaf_rem ? lo : m.leaf_rem);
             const uint64_t r1 = (hi + 1ull) * m.leaf_base + (hi + 1ull < m.leaf_rem ? hi + 1ull : m.leaf_rem) - 1;
-            const uint32_t s0 = div_by(static_cast<uint32_t>(r0 / G), w.span, m.span_inv), s1 = div_by(static_cast<uint32_t>(r1 / G), w.span, m.span_inv);
+            const uint32_t s0 = div_by(static_cast<uint32_t>(r0 / G), w.span, m.span_inv);
+            const uint32_t s1 = div_by(static_cast<uint32_t>(r1 / G), w.span, m.span_inv);
             // proven by the separators on both sides, else the whole top searched
             if ((s0 == 0 || sep[s0 - 1] < word) && (s1 + 1 >= w.segs || !(sep[s1] < word)))
                 seg = walk_segment_in<W>(sep, s0, s1, word);
@@ -582,7 +585,8 @@ static cudaError_t walk_launch(const bt_tree *t, const ModelDev *md, const void 
     auto kern = k_walk<K, V, MODEL>;
     const WalkDev &w = t->walk;
     constexpr int kMaxTop = walk_max_top(sizeof(K));
-    constexpr int kMaxModel = MODEL == kModelNone ? 0 : static_cast<int>(kModelSmemSegments) * 20 + 64 + static_cast<int>(kErrRanges) * 4;
+    constexpr int kMaxModel =
+        MODEL == kModelNone ? 0 : static_cast<int>(kModelSmemSegments) * 20 + 64 + static_cast<int>(kErrRanges) * 4;
     int sms = 0;
     cudaError_t e = dev_sm_count(&sms);
     if (e == cudaSuccess) e = ensure_dyn_smem(reinterpret_cast<const void *>(kern), kMaxTop + kMaxModel, kWalkCarveout);

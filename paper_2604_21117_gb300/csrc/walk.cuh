@@ -8,10 +8,9 @@
 // form that costs the fewest sectors per query:
 //
 //   top      the largest keys of up to 15360 segments of equal length (25600
-//            for 32-bit keys),
-//            ascending, and two tables that narrow the search
-//            among them to a few: the octave of x = key - smallest key (its
-//            leading one) gives a range of bins, as many as the octave has
+//            for 32-bit keys), ascending, and two tables that narrow the
+//            search among them to a few: the octave of x = key - smallest key
+//            (its leading one) gives a range of bins, as many as the octave has
 //            separators (rounded down to a power of two), the bits after the
 //            leading one a bin of them, and the bin the separators in it.  For
 //            uniform keys the upper octaves' bins hold one or two separators
@@ -206,7 +205,8 @@ __device__ __forceinline__ uint32_t walk_segment(const WalkDev &w, const unsigne
     uint64_t x;
     const uint32_t o = walk_octave<W>(w, q, x);
     const WalkOctave oct = reinterpret_cast<const WalkOctave *>(top + w.oct_off)[o];
-    const uint16_t *bins = reinterpret_cast<const uint16_t *>(top + w.bin_off) + oct.base + static_cast<uint32_t>(x >> oct.shift);
+    const uint32_t bin = oct.base + static_cast<uint32_t>(x >> oct.shift);
+    const uint16_t *bins = reinterpret_cast<const uint16_t *>(top + w.bin_off) + bin;
     return walk_segment_in<W>(reinterpret_cast<const W *>(top), bins[0], bins[1], q);
 }
 
