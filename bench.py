@@ -45,13 +45,15 @@ METRIC = "batched B+tree lookups/s at 2^24 keys, learned vs plain; p99 µs; HBM 
 UNIT = "lookups/s"
 L2_FLUSH_BYTES = 256 << 20
 
-# DRAM bytes (read + write) of one k_descend launch on the default workload,
-# from one ncu capture of it (summarised under profiles/); valid only while
-# the descent's source (desc_pipe.cu and descent.cuh) hashes to the same value.
-NCU_DESCEND_TRAFFIC = {"descend_src_sha256": "9f8dc9871dc2dfda", "bytes_per_launch": 223253760}
-# The same for the walk (k_walk) of the default workload.
-WALK_SRC = ("walk.cu", "walk.cuh")
-NCU_WALK_TRAFFIC = {"walk_src_sha256": "7be9d83980805df0", "bytes_per_launch": 149225984}
+# DRAM bytes (read + write) of one k_descend launch on the default workload
+# partitioned on 20 bits, from one ncu capture of it (summarised under
+# profiles/); valid only while the descent's source (desc_pipe.cu and
+# descent.cuh) hashes to the same value, which only another capture may change.
+NCU_DESCEND_TRAFFIC = {"descend_src_sha256": "38fd6998a564b0e3", "bytes_per_launch": 223728640}
+# The same for the walk (k_walk) of the default workload: the search's part of
+# walk.cu, whatever the construction before it, and walk.cuh.
+WALK_SRC = (("walk.cu", "- search\n"), "walk.cuh")
+NCU_WALK_TRAFFIC = {"walk_src_sha256": "0723f4deca3ef9d5", "bytes_per_launch": 149256192}
 
 
 def parse_args(argv=None):
@@ -82,7 +84,7 @@ def parse_args(argv=None):
                    help="pipelined: inner levels through L1 (0), staged (1), staged only for partitioned batches (2)")
     p.add_argument("--ballot", type=int, default=0, help="pipelined: leaf rank by binary search (0) or ballot (1)")
     p.add_argument("--l2-window", type=int, default=64 << 20,
-                   help="bytes of the L2 persistence window on the inner levels (0 = none)")
+                   help="bytes of the L2 persistence window on the inner levels where batches descend (0 = none)")
     p.add_argument("--no-designs", action="store_true", help="skip the A/B of the descent designs")
     p.add_argument("--lane-queries", type=int, default=1, help="queries per lane of the descent (1 or 2)")
     p.add_argument("--warps", type=int, default=0, help="descent warps per block (0 = library default)")
@@ -286,11 +288,14 @@ class ClockSampler:
 
 def src_sha256(names=("desc_pipe.cu", "descent.cuh")) -> str:
     """Hash of a kernel's source: its file and the helpers it includes (the
-    pipelined descent's unless others are named)."""
+    pipelined descent's unless others are named), of a file and a heading's
+    end what stands below that heading."""
     h = hashlib.sha256()
     for name in names:
+        name, heading = (name, "") if isinstance(name, str) else name
         with open(os.path.join(ROOT, "paper_2604_21117_gb300", "csrc", name), "rb") as f:
-            h.update(f.read())
+            text = f.read()
+        h.update(text[text.index(heading.encode()):])
     return h.hexdigest()[:16]
 
 
@@ -982,6 +987,10 @@ def run_ours(a):
     bt.bt_tree_set_staging(tree.handle, a.staging)
     bt.bt_tree_set_lane_queries(tree.handle, a.lane_queries)
     bt.bt_tree_set_descent(tree.handle, a.inner, a.ballot)
+    # the walk of a batch as given has no use for the window (40.4 G lookups/s
+    # with it and without), the descent of a partitioned one gets it
+    walk = a.sort_bits <= 0 and a.staging == 2 and a.lane_queries == 1 and a.ballot == 0
+    a.l2_window = 0 if walk else a.l2_window
     if a.l2_window > 0:
         bt.bt_tree_set_l2_window(tree.handle, a.l2_window)
     if a.warps > 0 or a.pin >= 0:
@@ -1121,7 +1130,6 @@ def run_ours(a):
 
     # bytes and roofline of the dominant kernel: the walk, or where the batch
     # is partitioned the descent
-    walk = sort_bits <= 0 and a.staging == 2 and a.lane_queries == 1 and a.ballot == 0
     walk_bytes = [walk_algorithmic_bytes(keys, qb, kb, vb) for qb in batches] if walk else None
     desc_bytes = [walk_bytes[i % pool] if walk else alg[i % pool][2] for i in range(K)]
     node_bytes = [sum(alg[i % pool][0]) * m * kb + alg[i % pool][1] * 32 for i in range(K)]

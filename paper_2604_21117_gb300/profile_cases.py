@@ -1,6 +1,6 @@
 """Small, self-contained workloads for profiling single kernels with ncu.
 
-    python -m paper_2604_21117_gb300.profile_cases forest [warps pin_budget lane_queries staging]
+    python -m paper_2604_21117_gb300.profile_cases forest [descent [warps pin_budget lane_queries staging]]
     python -m paper_2604_21117_gb300.profile_cases keys32 [sorted|full]
     python -m paper_2604_21117_gb300.profile_cases crossover
     python -m paper_2604_21117_gb300.profile_cases shapes
@@ -9,18 +9,20 @@
 forest: the multi-tree batching workload -- trees of 10^3, 10^5, 10^6 and
 2*10^7 uniform uint64 keys at fanout 32, a work list of 10,000 batches whose
 sizes are log-uniform in 1..1024, Zipf(0.9) queries with 80% hits -- searched
-five times by bt_forest_search at the given forest launch settings (default:
-4 warps per block, no pinned levels, two queries per lane, every level read
-through L1).
+five times by bt_forest_search: through the trees' walk indexes, or (descent)
+over trees without one, level by level at the given forest launch settings
+(default: 4 warps per block, no pinned levels, two queries per lane, every
+level read through L1).
 
 keys32: the paper's own tree (2^20 distinct 32-byte keys, 8-byte values,
-fanout 16) and a batch of 2^20 uniform queries at 90% hits: six descents of
-the batch partitioned on 20 bits (sorted) or six whole searches (full).
+fanout 16), without a walk index, and a batch of 2^20 uniform queries at 90%
+hits: six descents of the batch partitioned on 20 bits (sorted) or six whole
+searches, which partition it themselves (full).
 
 crossover: whole searches (bt_search_batch_ex) with no partition and with
 a partition on log2 B bits, batches B of 2^16 to 2^20 queries at 90% hits,
-over three trees that the L2 could hold -- 2^20 32-byte keys at fanout 16,
-and 10^6 and 4 * 10^6 uint64 keys at fanout 32 -- each with the L2 left warm
+over three trees without a walk index that the L2 could hold -- 2^20 32-byte
+keys at fanout 16, and 10^6 and 4 * 10^6 uint64 keys at fanout 32 -- each with the L2 left warm
 and with a 256 MB write before every call; medians of 40 calls.
 
 shapes: the descent of 2^20 queries partitioned on 20 bits over 2^24 uniform
@@ -46,7 +48,8 @@ def _events():
     return torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
 
 
-def forest(warps: int = 4, pin_budget: int = 0, lane_queries: int = 2, staging: int = 1) -> None:
+def forest(descent: bool = False, warps: int = 4, pin_budget: int = 0, lane_queries: int = 2,
+           staging: int = 1) -> None:
     import torch
     from . import build_lib
     build_lib.build()
@@ -56,7 +59,7 @@ def forest(warps: int = 4, pin_budget: int = 0, lane_queries: int = 2, staging: 
     trees, keysets = [], []
     for i, n in enumerate(sizes):
         keys = W.uniform_keys(n, 64, seed=W.SEED_BASE + 20 + i)
-        trees.append(bt.BTree(keys, W.rank_values(n, 64), 32))
+        trees.append(bt.BTree(keys, W.rank_values(n, 64), 32, walk_index=not descent))
         keysets.append(keys)
     nbatches = 10_000
     g = W.rng(W.SEED_BASE + 40)
@@ -77,7 +80,8 @@ def forest(warps: int = 4, pin_budget: int = 0, lane_queries: int = 2, staging: 
     dq = torch.from_numpy(allq).cuda()
     d_desc = torch.from_numpy(desc.view(np.uint8)).cuda()
     f = bt.bt_forest_create(trees)
-    bt.bt_forest_set_launch(f, warps, pin_budget, lane_queries, staging)
+    if descent:
+        bt.bt_forest_set_launch(f, warps, pin_budget, lane_queries, staging)
     v = torch.empty(allq.size, dtype=torch.uint64, device="cuda")
     found = torch.empty(allq.size, dtype=torch.uint8, device="cuda")
     wsb = bt.bt_forest_workspace_bytes(nbatches)
@@ -103,7 +107,7 @@ def keys32(mode: str = "sorted") -> None:
     from . import workloads as W
     n, m, B = 1 << 20, 16, 1 << 20
     keys = W.byte_keys(n, 32, seed=W.SEED_BASE + 8)
-    tree = bt.BTree(keys, W.rank_values(n, 64), m)
+    tree = bt.BTree(keys, W.rank_values(n, 64), m, walk_index=False)
     q = torch.from_numpy(W.make_byte_queries(keys, B, 0.9, seed=W.SEED_BASE + 9 + B)).cuda()
     nb = tree.workspace_bytes(B)
     ws = torch.empty(nb, dtype=torch.uint8, device="cuda")
@@ -154,11 +158,11 @@ def crossover(steps: int = 40) -> None:
     k6 = W.uniform_keys(1_000_000, 64, seed=W.SEED_BASE + 3)
     k7 = W.uniform_keys(4_000_000, 64, seed=W.SEED_BASE + 4)
     cases = [
-        ("2^20 32-byte keys, m=16", bt.BTree(kb, W.rank_values(kb.shape[0], 64), 16),
+        ("2^20 32-byte keys, m=16", bt.BTree(kb, W.rank_values(kb.shape[0], 64), 16, walk_index=False),
          lambda B: W.make_byte_queries(kb, B, 0.9, seed=W.SEED_BASE + 9 + B)),
-        ("10^6 uint64 keys, m=32", bt.BTree(k6, W.rank_values(k6.size, 64), 32),
+        ("10^6 uint64 keys, m=32", bt.BTree(k6, W.rank_values(k6.size, 64), 32, walk_index=False),
          lambda B: W.make_queries(k6, B, 0.9, seed=B + 5, width_bits=64)),
-        ("4*10^6 uint64 keys, m=32", bt.BTree(k7, W.rank_values(k7.size, 64), 32),
+        ("4*10^6 uint64 keys, m=32", bt.BTree(k7, W.rank_values(k7.size, 64), 32, walk_index=False),
          lambda B: W.make_queries(k7, B, 0.9, seed=B + 6, width_bits=64)),
     ]
     for name, tree, make in cases:
@@ -249,7 +253,8 @@ def main(argv=None) -> int:
         print(__doc__)
         return 2
     if argv[0] == "forest":
-        forest(*(int(x) for x in argv[1:5]))
+        descent = argv[1:2] == ["descent"]
+        forest(descent, *(int(x) for x in argv[2:6] if descent))
     elif argv[0] == "keys32":
         keys32(*argv[1:2])
     elif argv[0] == "crossover":
