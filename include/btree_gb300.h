@@ -331,8 +331,9 @@ uint64_t bt_search_host_workspace_bytes(const bt_tree *tree, uint64_t nq);
  * The call returns once the work is enqueued: synchronize `stream` before
  * reading h_out_vals / h_out_found.  Page-locked host buffers make the
  * copies asynchronous, and a batch that goes through the walk index reads
- * and writes them in place, without copies (queries that overlap the results
- * or lie off their alignment are copied); pageable ones work but the copies
+ * and writes them in place, without copies (queries that overlap the results,
+ * lie off their alignment or are not page-locked from the first byte to the
+ * last are copied); pageable ones work but the copies
  * then block.
  *
  *   h_queries, h_out_vals, h_out_found   host buffers of nq entries.
